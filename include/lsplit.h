@@ -194,7 +194,10 @@ int ls_init_gaussian(ls_ctx* ctx, void* psi_dev, const double* x0_host, double w
  * layer factor is one fused pass over the array.  Stochastic schemes apply
  * kinetic factors lazily and finish with a settle pass, so psi_dev is complete
  * on return.  With LS_MASK_PROJECT_EACH_STEP every step ends with the
- * projection onto the joint cutoff.  Enqueued on stream (replays a cached CUDA
+ * projection onto the joint cutoff.  Deterministic 1D calls with short
+ * potential kernels may alternate between psi_dev and a second array of the
+ * same size that the library allocates (one per psi_dev with cached graphs,
+ * freed with them; without memory for it the call runs in place).  Enqueued on stream (replays a cached CUDA
  * graph, one per (psi_dev, scheme, tau, nsteps); the graphs keep the tables
  * they use alive, and the table caches are bounded). */
 int ls_step(ls_ctx* ctx, void* psi_dev, int64_t nsteps, double tau, int32_t scheme,

@@ -155,6 +155,8 @@ struct CachedTab {
   // compact-kernel tables: the interaction-frame taps c'_d / (1 + c'_0)
   // (zero centre) and 1 + c'_0, the factor's scalar part
   std::shared_ptr<DevBuf> ipbuf;
+  std::vector<cd> iptaps;
+  double tail = 0;    // l1 norm of the dropped taps
   std::complex<double> diag{1.0, 0.0};
 };
 constexpr size_t kTableCacheCap = 48;
@@ -168,6 +170,7 @@ struct GraphEntry {
   int64_t n;
   cudaGraphExec_t exec = nullptr;
   std::shared_ptr<DevBuf> lists;
+  std::shared_ptr<DevBuf> alt;   // tile form: the second state array (shared by the graphs of one psi)
   TableKeep tables;  // every table the captured kernels read
   ~GraphEntry() {
     if (exec) cudaGraphExecDestroy(exec);
@@ -196,6 +199,7 @@ struct ls_ctx {
   bool fast2d[2] = {false, false};  // 64 x 64 slices on the fast 2D pass
   bool tc2d = false;                // layer-1 64 x 64 slices on the tensor-core pass
   DevBuf tcplanes;                  // its split-BF16 DFT matrix planes
+  DevBuf dir4, dir2;                // complex128 tile form: direction tables (built on first use)
   int sms = 0;
   int fast_variant = 0;   // shared-buffer / register-budget variant of the fast pass
   DevBuf tw[2], twb[2], bm[2], bp[2], chirp[2], vgrid[2];
@@ -397,6 +401,8 @@ CachedTab stencil_table(ls_ctx* c, int layer, double s) {
         upload_c(c, *e.buf, taps);
         e.ipbuf = std::make_shared<DevBuf>();
         upload_c(c, *e.ipbuf, iptaps);
+        e.iptaps = iptaps;
+        e.tail = tail;
         e.B = B;
         break;
       }
@@ -880,6 +886,210 @@ lsk::SamplerArgs sampler_args(ls_ctx* c, int scheme, int& npf) {
   return sa;
 }
 
+// ---- tile form of a deterministic compact-kernel call (lsplit_tile.cu)
+
+// Taps of one layer for the tile form: its half-width class (0: the layer does
+// not take the form), the taps split into float pairs.  complex128 forms the
+// correction in pairs of floats (2^-46 relative): the taps must sum to at most
+// 2^-7, so that this stays below an FP64 rounding of the result, and those
+// beyond |d| = 2 to single floats, at most 2^-30 each.
+int tile_taps(const ls_ctx* c, const CachedTab& t, float4* out) {
+  if (t.B <= 0 || t.iptaps.empty()) return 0;
+  const bool dbl = c->dtype == LS_C128;
+  if (t.B > (dbl ? 5 : 3)) return 0;
+  double sum = 0, far = 0;
+  for (int k = 0; k <= 2 * t.B; ++k) {
+    const double v = std::abs(t.iptaps[k]);
+    sum += v;
+    if (std::abs(k - t.B) >= 3) far = std::max(far, v);
+  }
+  if (!std::isfinite(sum) || (dbl && (sum > 0x1p-7 || far > 0x1p-30))) return 0;
+  // narrower by one where the l1 bound of the dropped taps still holds
+  // (stencil_table's classes jump from 3 to 5)
+  int B = t.B;
+  if (B == 5 && t.tail + std::abs(t.iptaps[0]) + std::abs(t.iptaps[10]) <= 0x1p-48) B = 4;
+  for (int k = 0; k <= 2 * t.B; ++k) {
+    const cd v = t.iptaps[k];
+    float4 f;
+    f.x = (float)v.real();
+    f.y = dbl ? (float)(v.real() - (double)f.x) : 0.f;
+    f.z = (float)v.imag();
+    f.w = dbl ? (float)(v.imag() - (double)f.z) : 0.f;
+    if (std::abs(k - t.B) <= B) out[lsk::kTileMaxB + k - t.B] = f;
+  }
+  return B;
+}
+
+// Factors per step, their layers and durations, and the kinetic units before
+// each of them and per step, of a deterministic scheme that the tile form takes.
+struct TileScheme {
+  int npf = 0;
+  int layer[3];
+  double s[3];
+  int64_t off[3], step = 0;
+};
+bool tile_scheme(int scheme, double tau, TileScheme& ts) {
+  if (scheme != LS_LIE && scheme != LS_STRANG && scheme != LS_STRANG_KP) return false;
+  std::vector<PassSpec> ps;
+  int32_t end = 0;
+  build_passes(scheme, tau, 1, ps, end);
+  ts.npf = (int)ps.size();
+  ts.step = end;
+  int64_t t = 0;
+  for (int i = 0; i < ts.npf; ++i) {
+    t += ps[i].pre;
+    ts.layer[i] = ps[i].layer;
+    ts.s[i] = ps[i].s;
+    ts.off[i] = t;
+    t += ps[i].post;
+  }
+  return true;
+}
+
+// Half-width class of the kernel for the given taps, 0 if the scheme or a
+// layer does not qualify; inst receives the taps, Lambda of n steps and the
+// geometry (set_kinetic's unit is the scheme's).
+int tile_instance(ls_ctx* c, int scheme, double tau, int64_t n, lsk::TileInst* inst) {
+  TileScheme ts;
+  if (c->d != 1 || c->mask_mode != LS_MASK_INIT_ONLY || !tile_scheme(scheme, tau, ts) || getenv_flag("LSPLIT_NO_IP") ||
+      getenv_flag("LSPLIT_NO_TILE"))
+    return 0;
+  // complex64: where the in-place passes are bound by their launches.  Up to
+  // about four 32 x 32 tiles per SM the tile form is faster (Strang, 20 steps,
+  // us: 33 x 33 100 against 191, 257 x 257 121 / 328, 513 x 513 205 / 350),
+  // beyond the halos cost more than the launches (769 x 769 381 / 343).
+  if (c->dtype == LS_C64 && c->M1 * c->M2 > (int64_t)c->sms * 4 * 24 * 28) return 0;
+  lsk::TileInst in;
+  std::memset(&in, 0, sizeof(in));
+  int bv = 0;
+  cd lam(1.0, 0.0);
+  for (int i = 0; i < ts.npf; ++i) {
+    const CachedTab t = stencil_table(c, ts.layer[i], ts.s[i]);
+    const int b = tile_taps(c, t, in.taps[ts.layer[i] - 1]);
+    if (b == 0) return 0;
+    bv = std::max(bv, b);
+    lam *= t.diag;
+  }
+  if (inst) {
+    lambda_parts(std::pow(lam, (double)n), in.lam_turns, in.lam_def);
+    in.pitch = c->pitch;
+    in.M1 = (int32_t)c->M1;
+    in.M2 = (int32_t)c->M2;
+    in.lo1 = c->geom[0].lo_a;
+    in.lo2 = c->geom[1].lo_a;
+    in.A1 = c->geom[0].A_aa;
+    in.A2 = c->geom[0].C_aa;
+    in.X = c->geom[0].X_aa;
+    *inst = in;
+  }
+  return std::max(bv, c->dtype == LS_C64 ? 2 : 3);
+}
+
+// The passes of n steps: an even number (the state ends in the caller's
+// array), nf factors each (two for nf = 1 where the count is odd), and the
+// halos and factors of every pass.
+std::vector<lsk::TileArgs> tile_passes(int scheme, double tau, int64_t n, int bv, int nf) {
+  TileScheme ts;
+  tile_scheme(scheme, tau, ts);
+  const int64_t F = n * ts.npf, P = std::min(2 * ((F + 2 * nf - 1) / (2 * nf)), F / 2 * 2);
+  std::vector<lsk::TileArgs> out;
+  out.reserve(P);
+  for (int64_t p = 0; p < P; ++p) {
+    lsk::TileArgs a;
+    std::memset(&a, 0, sizeof(a));
+    for (int64_t f = p * F / P; f < (p + 1) * F / P; ++f) {
+      const int r = (int)(f % ts.npf);
+      a.layer[a.nf] = ts.layer[r];
+      a.t[a.nf++] = (f / ts.npf) * ts.step + ts.off[r];
+      (ts.layer[r] == 1 ? a.hc : a.hr) += bv;
+    }
+    a.flip = (int)(p & 1);
+    a.last = p + 1 == P;
+    a.T = n * ts.step;
+    out.push_back(a);
+  }
+  return out;
+}
+
+int64_t tile_count(const ls_ctx* c, const lsk::TileArgs& a) {
+  return ((c->M2 + a.tr - 1) / a.tr) * ((c->M1 + a.tc - 1) / a.tc);
+}
+
+// Extent e of the tiles (with their halos) and factors per pass nf.
+// complex64: 32 x 32, a whole Strang step or two Lie or kinetic/potential
+// steps.  complex128: the pair with the least time, a pass costing 3.5 us and
+// 4 ns (64 x 64 tiles) or 8 ns (16 and 32: short segments load and split more
+// neighbours than they keep) per element and factor of the busiest SM's tiles,
+// plus 8 elements per row for the tables; rates measured on 65 x 65 and 1025 x
+// 1025 boxes (1025 x 1025, 20 Strang steps: 3.2 ms with 64, 6.8 ms with 32).
+struct TilePlan {
+  int e = 0, nf = 0;
+};
+TilePlan tile_plan(const ls_ctx* c, int scheme, double tau, int64_t n, int bv) {
+  if (c->dtype == LS_C64) return TilePlan{32, scheme == LS_STRANG ? 3 : 4};
+  TilePlan best;
+  double least = 0;
+  for (int e : {16, 32, 64})
+    for (int nf = 1; nf <= 3; ++nf) {
+      if (bv == 5 && e == 16) continue;
+      double t = 0;
+      bool fits = true;
+      for (lsk::TileArgs a : tile_passes(scheme, tau, n, bv, nf)) {
+        a.tr = e - 2 * a.hr;
+        a.tc = e - 2 * a.hc;
+        fits = fits && a.tr > 0 && a.tc > 0;
+        if (!fits) break;
+        t += 3500.0 + (e == 64 ? 4.0 : 8.0) * (double)((tile_count(c, a) + c->sms - 1) / c->sms) * a.nf * (e * e + 8 * e);
+      }
+      if (fits && (best.e == 0 || t < least)) {
+        best = TilePlan{e, nf};
+        least = t;
+      }
+    }
+  return best;
+}
+
+void tile_tables(ls_ctx* c) {
+  if (c->dtype != LS_C128 || c->dir2.p) return;
+  std::vector<float> t4(256 * 4);
+  std::vector<double> t2(1024 * 2);
+  for (int j = 0; j < 256; ++j) {
+    const double v[2] = {std::cos(2.0 * kPi * j / 256.0), std::sin(2.0 * kPi * j / 256.0)};
+    for (int k = 0; k < 2; ++k) {
+      t4[4 * j + 2 * k] = (float)v[k];
+      t4[4 * j + 2 * k + 1] = (float)(v[k] - (double)t4[4 * j + 2 * k]);
+    }
+  }
+  for (int j = 0; j < 1024; ++j) {
+    t2[2 * j] = std::cos(2.0 * kPi * j / 1024.0);
+    t2[2 * j + 1] = std::sin(2.0 * kPi * j / 1024.0);
+  }
+  c->dir4.alloc(t4.size() * sizeof(float));
+  LS_CUDA(cudaMemcpy(c->dir4.p, t4.data(), t4.size() * sizeof(float), cudaMemcpyHostToDevice));
+  c->dir2.alloc(t2.size() * sizeof(double));
+  LS_CUDA(cudaMemcpy(c->dir2.p, t2.data(), t2.size() * sizeof(double), cudaMemcpyHostToDevice));
+}
+
+void enqueue_tiles(ls_ctx* c, void* psi, void* alt, int64_t n, double tau, int scheme, cudaStream_t st) {
+  std::vector<PassSpec> ps;
+  int32_t end = 0;
+  set_kinetic(c, build_passes(scheme, tau, 1, ps, end));
+  lsk::TileInst in;
+  const int bv = tile_instance(c, scheme, tau, n, &in);
+  in.psi = psi;
+  in.alt = alt;
+  const TilePlan x = tile_plan(c, scheme, tau, n, bv);
+  for (lsk::TileArgs a : tile_passes(scheme, tau, n, bv, x.nf)) {
+    a.tr = x.e - 2 * a.hr;
+    a.tc = x.e - 2 * a.hc;
+    a.one = in;
+    a.ctab = static_cast<const float4*>(c->dir4.p);
+    a.ptab = static_cast<const double2*>(c->dir2.p);
+    if (c->dtype == LS_C64) LS_CUDA(lsk::launch_tile<float>(a, bv, x.e, tile_count(c, a), st));
+    else LS_CUDA(lsk::launch_tile<double>(a, bv, x.e, tile_count(c, a), st));
+  }
+}
+
 // Arguments of a Crank-Nicolson layer factor of duration s (Eq. (tsCN)):
 // potential band, Jacobi sweep count from the diagonal-dominance ratio, tile
 // shape.  Returns LS_OK or LS_ERR_INVALID with a message.
@@ -997,7 +1207,11 @@ int si_args(ls_ctx* c, double tau, lsk::SiArgs& a) {
 
 // Enqueue the whole call on stream st (used both for capture and direct runs).
 void enqueue_step(ls_ctx* c, void* psi, int64_t n, double tau, int scheme, cudaStream_t st,
-                  DevBuf* lists) {
+                  DevBuf* lists, void* alt) {
+  if (alt) {
+    enqueue_tiles(c, psi, alt, n, tau, scheme, st);
+    return;
+  }
   if (scheme == LS_SEMI_IMPLICIT || scheme == LS_RANDOM_BATCH) {
     // out of place, alternating between psi and the scratch array
     lsk::SiArgs a;
@@ -1517,11 +1731,28 @@ int ls_step(ls_ctx* c, void* psi, int64_t n, double tau, int32_t scheme, uint64_
         ~KeepScope() { c->keep = nullptr; }
       } ks{c};
       c->keep = &e->tables;
-      prepare_tables(c, n, tau, scheme);
+      if ((reinterpret_cast<uintptr_t>(psi) & 15) == 0 && tile_instance(c, scheme, tau, n, nullptr)) {
+        tile_tables(c);
+        // the second state array, one per psi (graphs of other arrays may run
+        // on other streams); without room for it the call runs in place
+        for (auto& g : c->graphs)
+          if (g->psi == psi && g->alt) e->alt = g->alt;
+        if (!e->alt) {
+          try {
+            e->alt = std::make_shared<DevBuf>();
+            e->alt->alloc((size_t)c->pitch * c->M2 * c->esize);
+          } catch (const CudaError& ce) {
+            e->alt.reset();
+            cudaGetLastError();
+            if (ce.e != cudaErrorMemoryAllocation) throw;
+          }
+        }
+      }
+      if (!e->alt) prepare_tables(c, n, tau, scheme);
       cudaGraph_t graph = nullptr;
       LS_CUDA(cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal));
       try {
-        enqueue_step(c, psi, n, tau, scheme, c->cap, e->lists.get());
+        enqueue_step(c, psi, n, tau, scheme, c->cap, e->lists.get(), e->alt ? e->alt->p : nullptr);
       } catch (...) {
         cudaStreamEndCapture(c->cap, &graph);
         if (graph) cudaGraphDestroy(graph);

@@ -161,6 +161,38 @@ template <typename Real> cudaError_t fast2d_prepare(size_t max_smem);
 template <typename Real> cudaError_t launch_stencil(const PassArgs& a, int64_t ntiles, cudaStream_t st);
 template <typename Real> size_t stencil_smem_bytes(const LayerGeom& g, int W, int B);
 template <typename Real> cudaError_t stencil_prepare(size_t max_smem);
+// Two-dimensional tiles (lsplit_tile.cu): several consecutive factors of a
+// deterministic compact-kernel call per pass, in the interaction frame.
+constexpr int kTileMaxB = 5;          // widest compact kernel of the tile form
+constexpr int kTileMaxF = 4;          // factors per pass
+struct TileInst {
+  void *psi, *alt;                    // the caller's array and the second one
+  int64_t pitch;
+  int32_t M1, M2, lo1, lo2;
+  uint64_t A1, A2, X;                 // kappa(m, n) = A1 m^2 + X m n + A2 n^2, turns per kinetic unit
+  uint64_t lam_turns;                 // Lambda of the call
+  double lam_def;
+  float4 taps[2][2 * kTileMaxB + 1];  // per layer, tap d at kTileMaxB + d: (re hi, re lo, im hi, im lo)
+};
+struct TileArgs {
+  TileInst one;                       // a single instance (inst NULL), or
+  const TileInst* inst;               // ninst of them with cumulative tile counts
+  const int32_t* cum;
+  int32_t ninst;
+  int32_t nf;                         // factors of this pass
+  int32_t layer[kTileMaxF];
+  int64_t t[kTileMaxF];               // kinetic units before each factor, from the start of the call
+  int32_t hr, hc;                     // halo rows and columns
+  int32_t tr, tc;                     // rows and columns of a tile's result
+  int32_t flip;                       // 0: psi -> alt, 1: alt -> psi
+  int32_t last;                       // apply Lambda K(T)
+  int64_t T;
+  const float4* ctab;                 // complex128: 256 directions as pairs of floats
+  const double2* ptab;                // complex128: 1024 directions
+};
+// bv: 2 or 3 (complex64), 3, 4 or 5 (complex128); ext: rows and columns of a
+// tile with its halos, 32 (complex64), 16, 32 or 64 (complex128; not 16 with bv 5)
+template <typename Real> cudaError_t launch_tile(const TileArgs& a, int bv, int ext, int64_t ntiles, cudaStream_t st);
 // Tensor-core layer pass for contiguous 64 x 64 slices (complex64, MODE_STEP,
 // optionally the fused second factor in T2): the DFTs as split-BF16 matrix
 // products.  planes: 4 x 64 x 64 bf16 (row-major) with W[p][k] =
