@@ -1462,6 +1462,49 @@ void elem_args(ls_ctx* c) {
   e.ecut = c->p.ecut;
 }
 
+// One-pass observables of a 1D box whose potentials have at most 8 harmonics
+// (of |h| below the box length, h and -h counted once) per layer.
+bool obs_args(const ls_ctx* c, const void* psi, const void* chi, lsk::ObsArgs& a) {
+  if (c->d != 1 || getenv_flag("LSPLIT_NO_OBS1D")) return false;
+  std::memset(&a, 0, sizeof(a));
+  a.psi = psi;
+  a.chi = chi;
+  a.pitch = c->pitch;
+  a.M1 = (int32_t)c->M1;
+  a.M2 = (int32_t)c->M2;
+  a.lo1 = c->p.lo1[0];
+  a.lo2 = c->p.lo2[0];
+  a.b1 = c->p.B1[0];
+  a.b2 = c->p.B2[0];
+  for (int L = 0; L < 2; ++L) {
+    const std::vector<int32_t>& h = L == 0 ? c->h1 : c->h2;
+    const std::vector<double>& v = L == 0 ? c->c1 : c->c2;
+    const int32_t q = c->geom[L].qa;
+    // on the grid of q points h counts modulo q, and Re sum_h v_h e_h is
+    // sum_h w_h e_h with w_h = (v_h + conj v_{-h}) / 2
+    std::map<int32_t, cd> w;
+    for (size_t t = 0; t < h.size(); ++t) {
+      const int32_t r = ((h[t] % q) + q) % q;
+      const cd z(v[2 * t], v[2 * t + 1]);
+      w[r] += 0.5 * z;
+      w[(q - r) % q] += 0.5 * std::conj(z);
+    }
+    for (const auto& e : w) {
+      const int32_t r = e.first;
+      if (r == 0) {
+        a.w0[L] = e.second.real();
+      } else if (2 * r <= q) {
+        if (a.nh[L] == lsk::kObsMaxH) return false;
+        const double f = 2 * r == q ? 0.5 : 1.0;   // its own conjugate
+        a.h[L][a.nh[L]] = r;
+        a.wr[L][a.nh[L]] = f * e.second.real();
+        a.wi[L][a.nh[L]++] = f * e.second.imag();
+      }
+    }
+  }
+  return true;
+}
+
 int64_t reduce_into(ls_ctx* c, int nparts, double* out_dev, cudaStream_t st) {
   LS_CUDA(lsk::launch_reduce((const double*)c->partials.p, nparts, lsk::kObsQ, out_dev, st));
   return 0;
@@ -1793,10 +1836,16 @@ int ls_observables(ls_ctx* c, const void* psi, const void* chi, ls_obs* out, voi
   return guarded([&]() -> int {
     cudaStream_t st = S(stream);
     double* res = (double*)c->result.p;
-    if (c->dtype == LS_C64) LS_CUDA(lsk::launch_elem_obs<float>(c->ea, psi, chi, (double*)c->partials.p, c->nblk_elem, st));
+    lsk::ObsArgs oa;
+    const bool one_pass = obs_args(c, psi, chi, oa);
+    if (one_pass) {
+      double* part = (double*)c->partials.p;
+      if (c->dtype == LS_C64) LS_CUDA(lsk::launch_obs1d<float>(oa, part, c->nblk_elem, st));
+      else LS_CUDA(lsk::launch_obs1d<double>(oa, part, c->nblk_elem, st));
+    } else if (c->dtype == LS_C64) LS_CUDA(lsk::launch_elem_obs<float>(c->ea, psi, chi, (double*)c->partials.p, c->nblk_elem, st));
     else LS_CUDA(lsk::launch_elem_obs<double>(c->ea, psi, chi, (double*)c->partials.p, c->nblk_elem, st));
     reduce_into(c, c->nblk_elem, res, st);
-    for (int L = 0; L < 2; ++L) {
+    for (int L = 0; L < 2 && !one_pass; ++L) {
       lsk::PassArgs a = base_args(c, L, const_cast<void*>(psi));
       a.mode = lsk::MODE_MEASURE;
       a.partials = (double*)c->partials.p;
@@ -1813,8 +1862,8 @@ int ls_observables(ls_ctx* c, const void* psi, const void* chi, ls_obs* out, voi
     out->kmean[1] = c->d > 1 ? h[3] : 0.0;
     out->overlap_re = chi ? h[4] : 0.0;
     out->overlap_im = chi ? h[5] : 0.0;
-    out->epot1 = h[8];
-    out->epot2 = h[9];
+    out->epot1 = one_pass ? h[6] : h[8];
+    out->epot2 = one_pass ? h[7] : h[9];
     out->energy = out->ekin + out->epot1 + out->epot2;
     return LS_OK;
   });

@@ -161,6 +161,19 @@ template <typename Real> cudaError_t fast2d_prepare(size_t max_smem);
 template <typename Real> cudaError_t launch_stencil(const PassArgs& a, int64_t ntiles, cudaStream_t st);
 template <typename Real> size_t stencil_smem_bytes(const LayerGeom& g, int W, int B);
 template <typename Real> cudaError_t stencil_prepare(size_t max_smem);
+// Observables of a 1D box in one pass (lsplit_obs.cu); partials as
+// launch_elem_obs, with the potential energies of the layers at 6 and 7.
+constexpr int kObsMaxH = 8;
+struct ObsArgs {
+  const void *psi, *chi;              // chi may be NULL
+  int64_t pitch;
+  int32_t M1, M2, lo1, lo2;
+  double b1, b2;                      // k = b1 m + b2 n
+  // v_j = w0 + 2 Re sum_k (wr + i wi)_k e^{2 pi i h_k x / L_j}, 0 < h_k < box length
+  double w0[2], wr[2][kObsMaxH], wi[2][kObsMaxH];
+  int32_t nh[2], h[2][kObsMaxH];
+};
+template <typename Real> cudaError_t launch_obs1d(const ObsArgs& a, double* partials, int nblocks, cudaStream_t st);
 // Two-dimensional tiles (lsplit_tile.cu): several consecutive factors of a
 // deterministic compact-kernel call per pass, in the interaction frame.
 constexpr int kTileMaxB = 5;          // widest compact kernel of the tile form

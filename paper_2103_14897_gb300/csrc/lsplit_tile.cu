@@ -41,23 +41,14 @@
 // single floats.  The pairs are scaled by the tile's largest exponent, so the
 // whole FP64 range is taken.
 #include "lsplit_kernels.cuh"
+#include "lsplit_pair.cuh"
 
 namespace lsk {
 namespace {
 
 // ---------------------------------------------------------------- pairs of floats
-struct DF { float h, l; };
 struct CDF { DF x, y; };
 
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-__device__ __forceinline__ DF quick(float h, float l) {
-  const float s = __fadd_rn(h, l);
-  return DF{s, __fsub_rn(l, __fsub_rn(s, h))};
-}
 // a b + c d (SUB: a b - c d)
 template <bool SUB> __device__ __forceinline__ DF dot2(DF a, DF b, DF c, DF d) {
   const float ch = SUB ? -c.h : c.h, cl = SUB ? -c.l : c.l;
