@@ -192,8 +192,9 @@ int ls_init_gaussian(ls_ctx* ctx, void* psi_dev, const double* x0_host, double w
  * seed and step0 fix the stochastic samples (sub-step g = (step0 + k) *
  * factors_per_step + factor index).  Adjacent kinetic factors are merged; each
  * layer factor is one fused pass over the array.  Stochastic schemes apply
- * kinetic factors lazily and finish with a settle pass, so psi_dev is complete
- * on return.  With LS_MASK_PROJECT_EACH_STEP every step ends with the
+ * kinetic factors lazily (or, complex64 with short potential kernels, once for
+ * the whole call) and finish with a settle pass, so psi_dev is complete on
+ * return.  With LS_MASK_PROJECT_EACH_STEP every step ends with the
  * projection onto the joint cutoff.  Deterministic 1D calls with short
  * potential kernels may alternate between psi_dev and a second array of the
  * same size that the library allocates (one per psi_dev with cached graphs,
@@ -279,6 +280,9 @@ int ls_batch_init_gaussian(ls_batch* batch, void* psi_dev, const double* x0_host
  * schemes: instance i draws its samples with seed + i (sub-step g as in
  * ls_step), the sampled-slice lists are drawn on the device in the same graph,
  * kinetic phases are applied lazily and a settle phase ends the call.
+ * complex64 stochastic calls whose factors all take the compact-kernel form
+ * run one launch per sub-step instead (in the same graph; no waits, so no
+ * LS_ERR_TIMEOUT, and nothing for the autotuner to choose).
  * Synchronises the stream to read the status: LS_ERR_TIMEOUT if a wait
  * expired (psi is then incomplete; the batch stays usable). */
 int ls_batch_step(ls_batch* batch, void* psi_dev, int64_t nsteps, double tau, int32_t scheme,

@@ -776,7 +776,7 @@ cudaError_t launch(ls_ctx* c, const lsk::PassArgs& a0, int L, int64_t nitems, cu
     return lsk::launch_tc2d(a0, c->tcplanes.p, (int)std::min<int64_t>(nitems, 2 * (int64_t)c->sms), st);
   if (a0.sB > 0 && (a0.mode == lsk::MODE_STEP || a0.mode == lsk::MODE_LAZY)) {
     lsk::PassArgs a = a0;
-    a.W = c->stW[L];
+    a.W = a.ip && a.list ? 1 : c->stW[L];   // sampled slices in the interaction frame: one per CTA
     a.strided = (L == 1) ? 1 : 0;
     const int64_t ntiles = (nitems + a.W - 1) / a.W;
     if (c->dtype == LS_C64) return lsk::launch_stencil<float>(a, ntiles, st);
@@ -1268,9 +1268,22 @@ void enqueue_step(ls_ctx* c, void* psi, int64_t n, double tau, int scheme, cudaS
   const bool stoch = scheme == LS_LIE_STOCH || scheme == LS_STRANG_STOCH;
   int npf = 0;
   lsk::SamplerArgs sa = sampler_args(c, scheme, npf);
+  // Stochastic schemes in the interaction frame (complex64, every factor in the
+  // compact-kernel form): the kinetic factors act on every element, so the
+  // frame is the same as the deterministic one; the sampled slices get their
+  // factors, scalar parts included, and K(T) ends the call.  Otherwise the
+  // pending phases are applied when a slice is sampled (touch times).
+  bool sip = stoch && c->d == 1 && c->dtype == LS_C64 && !getenv_flag("LSPLIT_NO_IP");
+  for (size_t i = 0; i < ps.size() && sip; ++i) {
+    const int64_t S = c->geom[ps[i].layer - 1].nslices;
+    const int32_t p = std::max<int32_t>(1, (int32_t)(S / c->frac_den));
+    sip = stencil_table(c, ps[i].layer, ps[i].s * (double)S / (double)p).B > 0;
+  }
   if (stoch) {
-    LS_CUDA(lsk::launch_zero_i32((int32_t*)c->touch_row.p, c->M2, st));
-    LS_CUDA(lsk::launch_zero_i32((int32_t*)c->touch_col.p, c->M1, st));
+    if (!sip) {
+      LS_CUDA(lsk::launch_zero_i32((int32_t*)c->touch_row.p, c->M2, st));
+      LS_CUDA(lsk::launch_zero_i32((int32_t*)c->touch_col.p, c->M1, st));
+    }
     LS_CUDA(lsk::launch_sampler(sa, (const uint64_t*)c->seedbuf.p, (int32_t)(n * npf), (int32_t*)lists->p, st));
   }
   // Adjacent layer-1 factors of consecutive Strang steps (separated by one
@@ -1379,6 +1392,13 @@ void enqueue_step(ls_ctx* c, void* psi, int64_t n, double tau, int scheme, cudaS
       }
       a.list = (const int32_t*)lists->p + (int64_t)i * sa.pmax;
       a.nlist = p;
+      if (sip) {
+        a.mode = lsk::MODE_STEP;
+        a.ip = 1;
+        t_acc += q.pre;
+        a.ip_t = t_acc;
+        t_acc += q.post;
+      }
       a.touch_own = (int32_t*)(L == 0 ? c->touch_row.p : c->touch_col.p);
       a.touch_other = (const int32_t*)(L == 0 ? c->touch_col.p : c->touch_row.p);
       a.now = q.now;
@@ -1390,7 +1410,11 @@ void enqueue_step(ls_ctx* c, void* psi, int64_t n, double tau, int scheme, cudaS
     // pending in the stochastic schemes and with the merged kinetic factors
     if (project && (i + 1 == ps.size() || ps[i + 1].step != q.step)) enqueue_project(c, psi, st);
   }
-  if (stoch) {
+  if (sip) {
+    lsk::PassArgs a = base_args(c, 0, psi);
+    a.units_pre = t_acc;
+    LS_CUDA(lsk::launch_kin_rows<float>(a, st));
+  } else if (stoch) {
     // settle: every element gets its pending kinetic phase up to end_time
     lsk::PassArgs a = base_args(c, 0, psi);
     a.mode = lsk::MODE_KIN;
@@ -1646,7 +1670,7 @@ int ls_create(const ls_problem* prob, ls_ctx** out) {
       const char* tf = std::getenv("LSPLIT_TRANSFORM");
       c->conv_form[L] = W > 0 && g.bluestein && !(tf && std::string(tf) == "bluestein");
     }
-    const size_t smax = (size_t)std::max(c->M1, c->M2) * 5;
+    const size_t smax = (size_t)std::max(c->M1, c->M2) * lsk::kSamplerBytes;
     if (smax > 48 * 1024) LS_CUDA(lsk::sampler_prepare(block_max));
     if (smax > (size_t)dev_max) throw CudaError{cudaErrorInvalidValue, "too many slices for the sampler"};
     elem_args(c.get());
@@ -2112,6 +2136,7 @@ struct ls_batch {
   size_t smem = 0;
   int blocks = 0;
   int device = 0;
+  int max_smem = 0;           // opt-in shared memory per CTA
   struct Cached {
     void* psi;
     int scheme;
@@ -2229,6 +2254,10 @@ std::unique_ptr<ls_batch::Cached> build_batch_graph(ls_batch* b, void* psi, int6
     // the end): that kernel's deterministic tile body is this form
     const bool ip = kind == 1 && !stoch && b->dtype == LS_C64 &&
                     (scheme == LS_LIE || scheme == LS_STRANG || scheme == LS_STRANG_KP);
+    // and so do the sampled slices of stochastic calls (launches per sub-step,
+    // K(T) as their settle phase)
+    const bool sip = kind == 1 && stoch && b->dtype == LS_C64;
+    size_t list_smem = 0;
     std::vector<std::complex<double>> lam(ninst, std::complex<double>(1.0, 0.0));
     int32_t ip_step = 0;
     if (ip) {
@@ -2272,6 +2301,14 @@ std::unique_ptr<ls_batch::Cached> build_batch_graph(ls_batch* b, void* psi, int6
           a.strided = L == 1 ? 1 : 0;
           a.fast_logn = 0;
           if (kind == 1) a.subtiles = b->subtiles1;
+          if (sip) {
+            // sampled slices: about 512 elements per 128-thread CTA
+            int w = 1;
+            while (w < 16 && 2 * w * c->geom[L].qa <= 512) w *= 2;
+            a.W = w;
+            a.subtiles = 1;
+            list_smem = std::max(list_smem, lsk::stencil_smem_bytes<float>(c->geom[L], w, stt.B));
+          }
           if (ip) {
             a.taps = stt.ipbuf->p;
             a.ip = 1;
@@ -2336,9 +2373,10 @@ std::unique_ptr<ls_batch::Cached> build_batch_graph(ls_batch* b, void* psi, int6
         a.touch_own = rows;
         a.touch_other = rows + c->M2;
         a.now = (int32_t)(et * n);
+        if (sip) a.units_pre = (int64_t)et * n;
         sargs[i] = a;
         scum[i] = acc;
-        acc += (c->M2 + a.W - 1) / a.W;
+        acc += sip ? lsk::kin_blocks(a.g) : (c->M2 + a.W - 1) / a.W;
       }
       scum[ninst] = acc;
       ba.settle_items = acc;
@@ -2439,12 +2477,25 @@ std::unique_ptr<ls_batch::Cached> build_batch_graph(ls_batch* b, void* psi, int6
     ba.kind = kind;
     cudaGraph_t graph = nullptr;
     LS_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-    cudaError_t ce = cudaMemsetAsync(b->counters.p, 0, (size_t)(ninst + 1) * sizeof(unsigned long long), b->cap);
-    if (ce == cudaSuccess && stoch) ce = cudaMemsetAsync(b->touch.p, 0, b->touch.bytes, b->cap);
+    cudaError_t ce = sip ? lsk::batch_list_prepare((size_t)b->max_smem)
+                         : cudaMemsetAsync(b->counters.p, 0, (size_t)(ninst + 1) * sizeof(unsigned long long), b->cap);
+    if (ce == cudaSuccess && stoch && !sip) ce = cudaMemsetAsync(b->touch.p, 0, b->touch.bytes, b->cap);
     if (ce == cudaSuccess && stoch)
       ce = lsk::launch_batch_sampler(sa, static_cast<const uint64_t*>(b->seedbuf.p), (int64_t)ninst * n * npass,
                                      static_cast<int32_t*>(e->lists->p), b->cap);
-    if (ce == cudaSuccess)
+    if (ce == cudaSuccess && sip) {
+      for (int64_t k = 0; k < n && ce == cudaSuccess; ++k) {
+        int64_t t = k * et;
+        for (int q = 0; q < npass && ce == cudaSuccess; ++q) {
+          t += ps[q].pre;
+          ce = lsk::launch_batch_list(ba.args + (size_t)q * ninst, ba.cum + (size_t)q * (ninst + 1), ninst,
+                                      ba.pass_items[q], k, t, list_smem, b->cap);
+          t += ps[q].post;
+        }
+      }
+      if (ce == cudaSuccess)
+        ce = lsk::launch_batch_kin(ba.settle_args, ba.settle_cum, ninst, ba.settle_items, b->cap);
+    } else if (ce == cudaSuccess)
       ce = b->dtype == LS_C64
                ? lsk::launch_batch<float>(ba, kind == 1 ? b->nthreads1 : b->nthreads,
                                           kind == 1 ? b->blocks1 : b->blocks, kind == 1 ? b->smem1 : b->smem, b->cap)
@@ -2536,6 +2587,7 @@ std::string tune_key(const ls_batch* b, double tau, int32_t scheme) {
 // LSPLIT_STENCIL_CFG, or the timeout test hook armed.
 void maybe_tune(ls_batch* b, void* psi, int64_t n, double tau, int32_t scheme, cudaStream_t st) {
   if (!b->tune || b->unmet || b->dtype != LS_C64 || !batch_all_compact(b, tau, scheme)) return;
+  if (scheme == LS_LIE_STOCH || scheme == LS_STRANG_STOCH) return;   // launches per sub-step: nothing to choose
   const std::string key = tune_key(b, tau, scheme);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -2696,6 +2748,7 @@ int ls_batch_create(const ls_problem* probs, int32_t count, ls_batch** out) {
     int dev_max = 0;
     LS_CUDA(cudaDeviceGetAttribute(&dev_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device));
     if (smem + 4096 > (size_t)dev_max) throw CudaError{cudaErrorInvalidValue, "batched tile exceeds shared memory"};
+    b->max_smem = dev_max;
     b->smem = smem;
     int per_sm = 0, per_sm1 = 0;
     b->minb = 3;
@@ -2721,8 +2774,8 @@ int ls_batch_create(const ls_problem* probs, int32_t count, ls_batch** out) {
     }
     b->touch.alloc((size_t)tt * sizeof(int32_t));
     b->seedbuf.alloc(2 * sizeof(uint64_t));
-    if ((size_t)smax * 5 > 48 * 1024) LS_CUDA(lsk::batch_sampler_prepare((size_t)dev_max));
-    if ((size_t)smax * 5 > (size_t)dev_max - 1024) throw CudaError{cudaErrorInvalidValue, "too many slices for the sampler"};
+    if ((size_t)smax * lsk::kSamplerBytes > 48 * 1024) LS_CUDA(lsk::batch_sampler_prepare((size_t)dev_max));
+    if ((size_t)smax * lsk::kSamplerBytes > (size_t)dev_max - 1024) throw CudaError{cudaErrorInvalidValue, "too many slices for the sampler"};
     b->counters.alloc((size_t)(count + 1) * sizeof(unsigned long long));
     b->status.alloc(sizeof(int32_t));
     LS_CUDA(cudaMemset(b->status.p, 0, sizeof(int32_t)));

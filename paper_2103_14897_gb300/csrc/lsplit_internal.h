@@ -140,6 +140,7 @@ struct SamplerArgs {
   int32_t pattern[4];
   uint64_t seed, g0;
 };
+constexpr int kSamplerBytes = 9;     // shared memory per slice of the sampler
 cudaError_t launch_sampler(const SamplerArgs& sa, const uint64_t* seed_g0_dev, int32_t count,
                            int32_t* out, cudaStream_t st);
 cudaError_t sampler_prepare(size_t smem);
@@ -159,6 +160,9 @@ template <typename Real> cudaError_t fast2d_prepare(size_t max_smem);
 // kStencilThreads threads; the tile (W slices with their wrap halos) sits in
 // shared memory.  W must be a power of two for strided slices.
 template <typename Real> cudaError_t launch_stencil(const PassArgs& a, int64_t ntiles, cudaStream_t st);
+// K(units_pre) on every row of a 1D box (complex64), in kin_blocks() CTAs.
+int64_t kin_blocks(const LayerGeom& g);
+template <typename Real> cudaError_t launch_kin_rows(const PassArgs& a, cudaStream_t st);
 template <typename Real> size_t stencil_smem_bytes(const LayerGeom& g, int W, int B);
 template <typename Real> cudaError_t stencil_prepare(size_t max_smem);
 // Observables of a 1D box in one pass (lsplit_obs.cu); partials as
@@ -271,6 +275,13 @@ struct BatchSamplerArgs {
   const int64_t* pass_off;  // [ninst * npf]
   int32_t npf, nsteps, Smax;
 };
+// Stochastic complex64 calls in the interaction frame: one sub-step (args and
+// cumulative tile counts of its pass; list of step `step`, frame at ip_t) or
+// the final K(T) on every instance.
+cudaError_t launch_batch_list(const PassArgs* args, const int64_t* cum, int ninst, int64_t blocks, int64_t step,
+                              int64_t ip_t, size_t smem, cudaStream_t st);
+cudaError_t launch_batch_kin(const PassArgs* args, const int64_t* cum, int ninst, int64_t blocks, cudaStream_t st);
+cudaError_t batch_list_prepare(size_t max_smem);
 cudaError_t launch_batch_sampler(const BatchSamplerArgs& sa, const uint64_t* seed_g0_dev, int64_t blocks,
                                  int32_t* out, cudaStream_t st);
 cudaError_t batch_sampler_prepare(size_t max_block);

@@ -387,12 +387,6 @@ __device__ __forceinline__ void sweep(typename A::E* sp, int step, const float4*
   __syncthreads();
 }
 
-// Programmatic dependent launch: the passes of a call follow one another, and
-// the next one may start (geometry, tables) while this one drains; it waits
-// for this one's results before it reads or writes any state.
-__device__ __forceinline__ void pass_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pass_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // ---------------------------------------------------------------- complex128
 template <int BV, int RE, int CE, int SEG, int MINB>
 __global__ void __launch_bounds__(RE * CE / SEG, MINB) tile_f64_kernel(const __grid_constant__ TileArgs a) {
@@ -831,17 +825,7 @@ template <typename K> cudaError_t launch_k(K k, const TileArgs& a, int threads, 
                                            cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)ntiles);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, a);
+  return launch_pdl(k, (unsigned)ntiles, threads, smem, st, a);
 }
 template <int BV, int RE, int CE, int SEG, int MINB>
 cudaError_t launch_f32(const TileArgs& a, int64_t ntiles, cudaStream_t st) {
