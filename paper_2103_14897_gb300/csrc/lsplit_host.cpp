@@ -196,7 +196,7 @@ struct ls_ctx {
   lsk::LayerGeom geom[2]{};
   int W[2] = {1, 1}, bpt[2] = {2, 2}, nt[2] = {64, 64};
   int fastW[2] = {0, 0};  // slices per CTA of the fast 1D pass (0: not applicable)
-  bool fast2d[2] = {false, false};  // 64 x 64 slices on the fast 2D pass
+  bool fast2d[2] = {false, false};  // 16 x 16, 32 x 32 and 64 x 64 slices on the fast 2D pass
   bool tc2d = false;                // layer-1 64 x 64 slices on the tensor-core pass
   DevBuf tcplanes;                  // its split-BF16 DFT matrix planes
   DevBuf dir4, dir2;                // complex128 tile form: direction tables (built on first use)
@@ -1640,7 +1640,7 @@ int ls_create(const ls_problem* prob, ls_ctx** out) {
     for (int L = 0; L < 2; ++L) {
       const lsk::LayerGeom& g = c->geom[L];
       const size_t sm = c->dtype == LS_C64 ? lsk::fast2d_smem_bytes<float>(g) : lsk::fast2d_smem_bytes<double>(g);
-      c->fast2d[L] = g.d == 2 && g.qa == 64 && g.qb == 64 && sm <= (size_t)dev_max && !getenv_flag("LSPLIT_NO_FAST") &&
+      c->fast2d[L] = g.d == 2 && g.qa == g.qb && (g.qa == 16 || g.qa == 32 || g.qa == 64) && sm <= (size_t)dev_max && !getenv_flag("LSPLIT_NO_FAST") &&
                      !c->p.shared;
     }
     for (int L = 0; L < 2; ++L) {

@@ -1088,61 +1088,71 @@ pass_fast_kernel(const PassArgs a) {
   fast_tile<Real, LOGN, MODE, NBUF, FUSED, false>(a, (int64_t)blockIdx.x, smraw);
 }
 
-// ---------------------------------------------------------------- fast 2D pass (64 x 64 slices)
-// One 64 x 64 slice per 256-thread CTA.  The slice sits in shared memory with
-// row stride 65 (element (ia, ib) at ia + 65 ib).  A 64-point transform along
-// either axis is done by four threads: thread t takes line sub = t & 63 and
-// quarter j = t >> 6 and holds elements j + 4u + 8r (u < 2, r < 8) of the line
-// in v[8u + r].  All lanes of a warp share j and take 32 consecutive lines, so
-// every shared-memory access of both axes is free of bank conflicts.  Two
-// radix-8 Stockham stages; the output lands in the input layout, so the
-// inverse transform along b, the potential factor and the forward transform
-// along b follow one another in registers.
-constexpr int kF2Row = 65;
+// ---------------------------------------------------------------- fast 2D pass (N x N slices)
+// Slices of N x N points, N = 16, 32 or 64, in shared memory at row stride
+// N + 4 (element (ia, ib) at ia + (N + 4) ib).  A transform of a line, along
+// either axis, is done by four adjacent lanes: lane j of the four holds the
+// elements j + 4k (k < N/4), two Stockham stages (radix 8 x 8, 8 x 4, 4 x 4)
+// exchange within the line, so inside a transform only the warp synchronises;
+// the CTA does between the axes, three times per factor.  32 x 32 slices (the
+// 32^4 box, 10 Strang steps) took 1116 us on the general pass and take 312 us;
+// 64 x 64 slices take 16 % fewer instructions than with a quarter of the line
+// per warp and thirteen barriers, and the same time (MIO and FMA queues).
+// A half warp covers four lines; stride N + 4 = 4 modulo 16 puts its accesses
+// on distinct banks along both axes.
+template <int N> struct F2 {
+  static constexpr int kRow = N + 4, kE = N / 4, kThreads = 4 * N;
+  static constexpr int kR1 = N == 16 ? 4 : 8, kR2 = N / kR1;
+};
 
-template <typename Real, bool INV>
-__device__ __forceinline__ void fft64_line(typename CT<Real>::C (&v)[16], typename CT<Real>::C* buf, int base,
-                                           int es, int j, const typename CT<Real>::C* __restrict__ tw) {
+template <typename Real, bool INV, int N>
+__device__ __forceinline__ void fft_quad(typename CT<Real>::C (&v)[N / 4], typename CT<Real>::C* buf, int base, int es,
+                                         int j, const typename CT<Real>::C* __restrict__ tw) {
   using C = typename CT<Real>::C;
-  C wb[2];
+  constexpr int E = N / 4, R1 = F2<N>::kR1, R2 = F2<N>::kR2, U1 = E / R1, U2 = E / R2;
+  C wb[U2];
 #pragma unroll
-  for (int u = 0; u < 2; ++u) wb[u] = tw[j + 4 * u];  // W_64^b, b = j + 4u (stage 2, stride 1)
-  // stage 1 (ns = 1): butterfly b = j + 4u reads x[b + 8r], writes 8b + r
+  for (int u = 0; u < U2; ++u) wb[u] = tw[j + 4 * u];   // W_N^b of the second stage
+  // the exchange keeps index i at i ^ (i / R1 mod 4): with either the R1 (j + 4u)
+  // + r of the writes or the j + 4u + r N/R2 of the reads, the four lanes of a
+  // line then differ modulo 4, and the half warp's accesses fall on distinct banks
+  int q[4];
 #pragma unroll
-  for (int u = 0; u < 2; ++u) dftR<8, C, INV>(v + 8 * u);
+  for (int k = 0; k < 4; ++k) q[k] = base + (j ^ k) * es;
+  // stage 1: butterfly b = j + 4u reads x[b + r N/R1], writes R1 b + r
+  C t[R1];
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
+  for (int u = 0; u < U1; ++u) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r) buf[base + (8 * (j + 4 * u) + r) * es] = v[8 * u + r];
-  __syncthreads();
-  // stage 2 (ns = 8): butterfly b reads x[b + 8r], twiddles W_64^(r b), writes b + 8r
+    for (int r = 0; r < R1; ++r) t[r] = v[u + U1 * r];
+    dftR<R1, C, INV>(t);
+    if (u == 0) __syncwarp();   // every lane of the line has read its elements
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
+    for (int r = 0; r < R1; ++r) buf[q[r & 3] + (R1 * (j + 4 * u) + (r & ~3)) * es] = t[r];
+  }
+  __syncwarp();
+  // stage 2: butterfly b = j + 4u reads x[b + r N/R2], twiddles W_N^(r b), writes b + r R1
+  C z[U2 * R2];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) v[8 * u + r] = buf[base + (j + 4 * u + 8 * r) * es];
-  __syncthreads();
+  for (int u = 0; u < U2; ++u)
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    twiddle_pow<8, Real, INV>(v + 8 * u, wb[u]);
-    dftR<8, C, INV>(v + 8 * u);
+    for (int r = 0; r < R2; ++r) z[u * R2 + r] = buf[q[r & 3] + (4 * u + r * (N / R2)) * es];
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < U2; ++u) {
+    twiddle_pow<R2, Real, INV>(z + u * R2, wb[u]);
+    dftR<R2, C, INV>(z + u * R2);
+#pragma unroll
+    for (int r = 0; r < R2; ++r) v[u + U2 * r] = z[u * R2 + r];
   }
 }
-
-template <typename Real>
-__device__ __forceinline__ void f2_line_load(typename CT<Real>::C (&v)[16], const typename CT<Real>::C* buf,
-                                             int base, int es, int j) {
+template <typename C, int E> __device__ __forceinline__ void quad_load(C (&v)[E], const C* buf, int base, int es, int j) {
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[8 * u + r] = buf[base + (j + 4 * u + 8 * r) * es];
+  for (int k = 0; k < E; ++k) v[k] = buf[base + (j + 4 * k) * es];
 }
-template <typename Real>
-__device__ __forceinline__ void f2_line_store(const typename CT<Real>::C (&v)[16], typename CT<Real>::C* buf,
-                                              int base, int es, int j) {
+template <typename C, int E> __device__ __forceinline__ void quad_store(const C (&v)[E], C* buf, int base, int es, int j) {
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
-#pragma unroll
-    for (int r = 0; r < 8; ++r) buf[base + (j + 4 * u + 8 * r) * es] = v[8 * u + r];
+  for (int k = 0; k < E; ++k) buf[base + (j + 4 * k) * es] = v[k];
 }
 
 // Kinetic phase turns of one thread's elements (ia fixed, ib = ib0 + 4m,
@@ -1168,156 +1178,148 @@ struct QuadWalk {
   }
 };
 
-// The correction F diag((T - 1)/M) F^{-1} x of one slice held in buf (row
-// stride 65), in place: inverse transforms along a and b, the potential
-// factor, forward transforms along b and a.  Ends with a barrier.
-template <typename Real>
+// The correction F diag((T - 1)/M) F^{-1} x of one slice held in buf, in
+// place: inverse transforms along a and b, the potential factor, forward
+// transforms along b and a.  Thread r of the slice's 4 N takes line r / 4.
+// Called after a CTA barrier, ends with one.
+template <typename Real, int N>
 __device__ __forceinline__ void f2_correction(typename CT<Real>::C* buf, const typename CT<Real>::C* __restrict__ T,
                                               const typename CT<Real>::C* __restrict__ twa,
-                                              const typename CT<Real>::C* __restrict__ twb, int sub, int j) {
+                                              const typename CT<Real>::C* __restrict__ twb, int r) {
   using C = typename CT<Real>::C;
-  C v[16];
+  constexpr int E = N / 4, RS = F2<N>::kRow;
+  const int sub = r >> 2, j = r & 3;
+  C v[E];
   // inverse transform along a (line = row ib = sub)
-  f2_line_load<Real>(v, buf, sub * kF2Row, 1, j);
-  __syncthreads();
-  fft64_line<Real, true>(v, buf, sub * kF2Row, 1, j, twa);
-  f2_line_store<Real>(v, buf, sub * kF2Row, 1, j);
+  quad_load(v, buf, sub * RS, 1, j);
+  fft_quad<Real, true, N>(v, buf, sub * RS, 1, j, twa);
+  quad_store(v, buf, sub * RS, 1, j);
   __syncthreads();
   // inverse along b (line = column ia = sub), potential factor, forward along b
-  f2_line_load<Real>(v, buf, sub, kF2Row, j);
-  __syncthreads();
-  fft64_line<Real, true>(v, buf, sub, kF2Row, j, twb);
+  quad_load(v, buf, sub, RS, j);
+  fft_quad<Real, true, N>(v, buf, sub, RS, j, twb);
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[8 * u + r] = cmul(v[8 * u + r], T[sub + 64 * (j + 4 * u + 8 * r)]);
-  fft64_line<Real, false>(v, buf, sub, kF2Row, j, twb);
-  f2_line_store<Real>(v, buf, sub, kF2Row, j);
+  for (int k = 0; k < E; ++k) v[k] = cmul(v[k], T[sub + N * (j + 4 * k)]);
+  fft_quad<Real, false, N>(v, buf, sub, RS, j, twb);
+  quad_store(v, buf, sub, RS, j);
   __syncthreads();
   // forward along a
-  f2_line_load<Real>(v, buf, sub * kF2Row, 1, j);
-  __syncthreads();
-  fft64_line<Real, false>(v, buf, sub * kF2Row, 1, j, twa);
-  f2_line_store<Real>(v, buf, sub * kF2Row, 1, j);
+  quad_load(v, buf, sub * RS, 1, j);
+  fft_quad<Real, false, N>(v, buf, sub * RS, 1, j, twa);
+  quad_store(v, buf, sub * RS, 1, j);
   __syncthreads();
 }
 
-// FUSED: two layer-1 factors of consecutive Strang steps in one launch, with
-// the merged kinetic factor (units_mid) between them and the second factor's
-// table in T2; the intermediate slice stays in shared memory.
-template <typename Real, int MODE, bool FUSED = false>
-__global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 3 : 1)
-pass_fast2d_kernel(const PassArgs a) {
+// SP slices per CTA of SP 4 N threads.  For loads and stores thread t takes
+// elements ia, ib = j + 4m of a slice, consecutive threads consecutive ia
+// (contiguous layer) or consecutive slices (STRIDED, the layer whose slices
+// are adjacent in memory).  The identity term x stays in registers, for N = 64
+// in shared memory.  FUSED: two layer-1 factors of consecutive Strang steps in
+// one launch, with the merged kinetic factor (units_mid) between them and the
+// second factor's table in T2.
+template <typename Real, int MODE, bool FUSED, int N, int SP, bool STRIDED, int MINB>
+__global__ void __launch_bounds__(SP * 4 * N, MINB) pass_fast2d_kernel(const PassArgs a) {
   using C = typename CT<Real>::C;
   constexpr bool lazy = (MODE == MODE_LAZY);
+  constexpr bool REGS = N < 64;
+  constexpr int E = N / 4, RS = F2<N>::kRow, TS = F2<N>::kThreads;
+  // strided: buffers 4 elements apart modulo 16, so that the four slices of a
+  // half warp fall on distinct banks in the loads and stores
+  constexpr int SB = N * RS + (STRIDED ? 4 : 0);
   extern __shared__ __align__(16) unsigned char smraw[];
   const LayerGeom& g = a.g;
   const int t = threadIdx.x;
-  const int sub = t & 63, j = t >> 6;
+  const int lw = STRIDED ? t % SP : t / TS, lr = STRIDED ? t / SP : t % TS;
+  const int ia = lr % N, j = lr / N;
   C* buf = reinterpret_cast<C*>(smraw);
-  C* xs = buf + 64 * kF2Row;
-  __shared__ int64_t s_slice;
-  __shared__ uint64_t s_la, s_lb, s_c0;
-  __shared__ int32_t s_touch;
-  if (t == 0) {
-    int64_t s = -1;
-    if (a.list) {
-      if ((int64_t)blockIdx.x < a.nlist) s = a.list[blockIdx.x];
-    } else {
-      s = blockIdx.x;
-      if (s >= g.nslices) s = -1;
-    }
-    s_slice = s;
-    uint64_t la = 0, lb = 0, c0 = 0;
-    int32_t touch = 0;
-    if (s >= 0) {
-      const uint64_t ua = (uint64_t)(s % g.oqa + g.olo_a), ub = (uint64_t)(s / g.oqa + g.olo_b);
-      la = g.X_aa * ua + g.X_ab * ub;
-      lb = g.X_ba * ua + g.X_bb * ub;
-      c0 = g.C_aa * (ua * ua) + g.C_ab * (ua * ub) + g.C_bb * (ub * ub);
-      if (lazy) touch = a.touch_own[s];
-    }
-    s_la = la;
-    s_lb = lb;
-    s_c0 = c0;
-    s_touch = touch;
+  C* lb = buf + lw * SB;                 // this thread's slice in the loads and stores
+  C* xs = buf + SP * SB + (size_t)lw * N * N;
+  int64_t s = (int64_t)blockIdx.x * SP + lw;
+  if (a.list) s = s < a.nlist ? (int64_t)a.list[s] : -1;
+  else if (s >= g.nslices) s = -1;
+  uint64_t la = 0, lbb = 0, c0 = 0;
+  int32_t touch = 0;
+  if (s >= 0) {
+    const uint64_t ua = (uint64_t)(s % g.oqa + g.olo_a), ub = (uint64_t)(s / g.oqa + g.olo_b);
+    la = g.X_aa * ua + g.X_ab * ub;
+    lbb = g.X_ba * ua + g.X_bb * ub;
+    c0 = g.C_aa * (ua * ua) + g.C_ab * (ua * ub) + g.C_bb * (ub * ub);
+    if (lazy) touch = a.touch_own[s];
   }
-  __syncthreads();
-  const int64_t s = s_slice;
-  if (s < 0) return;
-  C* psi = reinterpret_cast<C*>(a.psi);
   const C* twa = reinterpret_cast<const C*>(g.tw);
   const C* twb = reinterpret_cast<const C*>(g.twb);
-  // this thread's elements in the load and store loops: ia = sub, ib = j + 4m
-  C* pp = psi + s * g.slice_stride + sub * g.ea + j * g.eb;
+  C* pp = reinterpret_cast<C*>(a.psi) + (s >= 0 ? s : 0) * g.slice_stride + ia * g.ea + j * g.eb;
   const int64_t estep = 4 * g.eb;
-  {
-    C x[16];
+  C x[E];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) x[m] = pp[m * estep];  // all loads in flight before the phases
-    if (lazy) {
-      QuadWalk w(g, sub, j, s_la, s_lb, s_c0);
+  for (int m = 0; m < E; ++m) x[m] = s >= 0 ? pp[m * estep] : czero<C>();   // all loads in flight before the phases
+  if (lazy) {
+    QuadWalk w(g, ia, j, la, lbb, c0);
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
-        const int32_t t2 = a.touch_other[sub + 64 * (j + 4 * m)];
-        const int64_t units = (int64_t)a.now - (int64_t)(s_touch > t2 ? s_touch : t2);
-        if (units != 0) x[m] = apply_phase<Real>(x[m], phase_of<Real>((uint64_t)0 - (uint64_t)units * w.q));
-        w.next();
-      }
-    } else if (a.units_pre != 0) {
-      QuadWalk w(g, sub, j, s_la, s_lb, s_c0);
-      w.scale((uint64_t)0 - (uint64_t)a.units_pre);
-#pragma unroll
-      for (int m = 0; m < 16; ++m) {
-        x[m] = apply_phase<Real>(x[m], phase_of<Real>(w.q));
-        w.next();
-      }
+    for (int m = 0; m < E; ++m) {
+      const int32_t t2 = a.touch_other[ia + N * (j + 4 * m)];
+      const int64_t units = (int64_t)a.now - (int64_t)(touch > t2 ? touch : t2);
+      if (units != 0) x[m] = apply_phase<Real>(x[m], phase_of<Real>((uint64_t)0 - (uint64_t)units * w.q));
+      w.next();
     }
+  } else if (a.units_pre != 0) {
+    QuadWalk w(g, ia, j, la, lbb, c0);
+    w.scale((uint64_t)0 - (uint64_t)a.units_pre);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      const int ib = j + 4 * m;
-      xs[sub + 64 * ib] = x[m];
-      buf[sub + kF2Row * ib] = x[m];
+    for (int m = 0; m < E; ++m) {
+      x[m] = apply_phase<Real>(x[m], phase_of<Real>(w.q));
+      w.next();
     }
   }
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int ib = j + 4 * m;
+    if constexpr (!REGS) xs[ia + N * ib] = x[m];
+    lb[ia + RS * ib] = x[m];
+  }
   __syncthreads();
-  f2_correction<Real>(buf, reinterpret_cast<const C*>(a.T), twa, twb, sub, j);
+  C* fb = buf + (t / TS) * SB;           // this thread's slice in the transforms
+  f2_correction<Real, N>(fb, reinterpret_cast<const C*>(a.T), twa, twb, t % TS);
+  auto sum = [&](int m) {                // x + correction
+    const int ib = j + 4 * m;
+    return cadd(REGS ? x[m] : xs[ia + N * ib], lb[ia + RS * ib]);
+  };
   if constexpr (FUSED) {
     // x1 = K(mid) (x + correction): the second factor's input and identity term
-    QuadWalk w(g, sub, j, s_la, s_lb, s_c0);
+    QuadWalk w(g, ia, j, la, lbb, c0);
     const bool mid = a.units_mid != 0;
     if (mid) w.scale((uint64_t)0 - (uint64_t)a.units_mid);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
+    for (int m = 0; m < E; ++m) {
       const int ib = j + 4 * m;
-      C x = cadd(xs[sub + 64 * ib], buf[sub + kF2Row * ib]);
+      C y = sum(m);
       if (mid) {
-        x = apply_phase<Real>(x, phase_of<Real>(w.q));
+        y = apply_phase<Real>(y, phase_of<Real>(w.q));
         w.next();
       }
-      xs[sub + 64 * ib] = x;
-      buf[sub + kF2Row * ib] = x;
+      if constexpr (REGS) x[m] = y;
+      else xs[ia + N * ib] = y;
+      lb[ia + RS * ib] = y;
     }
     __syncthreads();
-    f2_correction<Real>(buf, reinterpret_cast<const C*>(a.T2), twa, twb, sub, j);
+    f2_correction<Real, N>(fb, reinterpret_cast<const C*>(a.T2), twa, twb, t % TS);
   }
   // x + correction, kinetic post-phase, store
   {
     const bool post = !lazy && a.units_post != 0;
-    QuadWalk w(g, sub, j, s_la, s_lb, s_c0);
+    QuadWalk w(g, ia, j, la, lbb, c0);
     if (post) w.scale((uint64_t)0 - (uint64_t)a.units_post);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      const int ib = j + 4 * m;
-      C x = cadd(xs[sub + 64 * ib], buf[sub + kF2Row * ib]);
+    for (int m = 0; m < E; ++m) {
+      C y = sum(m);
       if (post) {
-        x = apply_phase<Real>(x, phase_of<Real>(w.q));
+        y = apply_phase<Real>(y, phase_of<Real>(w.q));
         w.next();
       }
-      pp[m * estep] = x;
+      if (s >= 0) pp[m * estep] = y;
     }
   }
-  if (lazy && t == 0) a.touch_own[s] = a.now;
+  if (lazy && lr == 0 && s >= 0) a.touch_own[s] = a.now;
 }
 
 // Two adjacent slices per CTA for the strided layer (slice stride 1 element):
@@ -1335,7 +1337,8 @@ __global__ void __launch_bounds__(256, 2) pass_fast2d_pair_kernel(const PassArgs
   const int t = threadIdx.x;
   const int sub = t & 63, j = t >> 6;
   C* buf = reinterpret_cast<C*>(smraw);
-  C* xs = buf + 64 * kF2Row;
+  constexpr int RS = F2<64>::kRow;
+  C* xs = buf + 64 * RS;
   __shared__ uint64_t s_la[2], s_lb[2], s_c0[2];
   const int64_t s0 = 2 * (int64_t)blockIdx.x;
   if (s0 >= g.nslices) return;
@@ -1386,11 +1389,11 @@ __global__ void __launch_bounds__(256, 2) pass_fast2d_pair_kernel(const PassArgs
     for (int m = 0; m < 16; ++m) {
       const int ib = j + 4 * m;
       xs[sub + 64 * ib] = x0[m];
-      buf[sub + kF2Row * ib] = x0[m];
+      buf[sub + RS * ib] = x0[m];
     }
   }
   __syncthreads();
-  f2_correction<float>(buf, T, twa, twb, sub, j);
+  f2_correction<float, 64>(buf, T, twa, twb, t);
   // first slice: x + correction, post-phase, kept in xs; second slice's input
   // into buf (each thread touches only its own elements here)
   {
@@ -1400,17 +1403,17 @@ __global__ void __launch_bounds__(256, 2) pass_fast2d_pair_kernel(const PassArgs
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int ib = j + 4 * m;
-      C x = cadd(xs[sub + 64 * ib], buf[sub + kF2Row * ib]);
+      C x = cadd(xs[sub + 64 * ib], buf[sub + RS * ib]);
       if (post) {
         x = apply_phase<float>(x, phase_of<float>(w.q));
         w.next();
       }
       xs[sub + 64 * ib] = x;
-      buf[sub + kF2Row * ib] = x1[m];
+      buf[sub + RS * ib] = x1[m];
     }
   }
   __syncthreads();
-  f2_correction<float>(buf, T, twa, twb, sub, j);
+  f2_correction<float, 64>(buf, T, twa, twb, t);
   {
     QuadWalk w(g, sub, j, s_la[1], s_lb[1], s_c0[1]);
     const bool post = a.units_post != 0;
@@ -1418,7 +1421,7 @@ __global__ void __launch_bounds__(256, 2) pass_fast2d_pair_kernel(const PassArgs
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int ib = j + 4 * m;
-      C x = cadd(x1[m], buf[sub + kF2Row * ib]);
+      C x = cadd(x1[m], buf[sub + RS * ib]);
       if (post) {
         x = apply_phase<float>(x, phase_of<float>(w.q));
         w.next();
@@ -1430,37 +1433,82 @@ __global__ void __launch_bounds__(256, 2) pass_fast2d_pair_kernel(const PassArgs
   }
 }
 
+// Slices per CTA: contiguous layer and lists (CTAs of 128 or 256 threads), and
+// the strided layer (4 or 8 adjacent slices: 32- or 64-byte segments).
+template <int N> struct F2Slices {
+  static constexpr int kC = N == 64 ? 1 : N == 32 ? 1 : 4, kS = N == 64 ? 1 : N == 32 ? 4 : 8;
+};
+template <typename Real, int MODE, bool FUSED, int N, int SP, bool STRIDED>
+static constexpr size_t f2_smem() {
+  return ((size_t)SP * (N * F2<N>::kRow + (STRIDED ? 4 : 0)) + (N == 64 ? (size_t)N * N : 0)) *
+         sizeof(typename CT<Real>::C);
+}
+// CTAs per SM the registers are budgeted for
+template <typename Real, int N, int SP> constexpr int f2_minb() {
+  return sizeof(Real) == 8 ? (N == 64 ? 1 : (SP * 4 * N > 256 ? 1 : 2)) : (N == 64 ? 3 : (1024 / (SP * 4 * N)));
+}
+#define LS_F2K(MODE, FUSED, N, SP, ST) pass_fast2d_kernel<Real, MODE, FUSED, N, SP, ST, f2_minb<Real, N, SP>()>
+
 template <typename Real> size_t fast2d_smem_bytes(const LayerGeom& g) {
-  using C = typename CT<Real>::C;
-  return ((size_t)64 * kF2Row + (size_t)g.M) * sizeof(C);
+  return g.qa == 64 ? f2_smem<Real, MODE_STEP, false, 64, 1, false>() : (size_t)0;   // the smaller ones always fit
 }
 
-template <typename Real> cudaError_t launch_fast2d(const PassArgs& a, int64_t ntiles, cudaStream_t st) {
-  if (ntiles <= 0) return cudaSuccess;
-  if (a.g.d != 2 || a.g.qa != 64 || a.g.qb != 64) return cudaErrorInvalidValue;
-  const size_t smem = fast2d_smem_bytes<Real>(a.g);
-  if constexpr (sizeof(Real) == 4) {
+template <typename Real, int N> static cudaError_t launch_fast2d_n(const PassArgs& a, int64_t n, cudaStream_t st) {
+  constexpr int SC = F2Slices<N>::kC, SS = F2Slices<N>::kS;
+  const unsigned bc = (unsigned)((n + SC - 1) / SC);
+  if constexpr (N == 64 && sizeof(Real) == 4) {
     // strided layer, full pass, 16-byte aligned slice pairs: two slices per CTA
     if (a.mode == MODE_STEP && a.list == nullptr && a.T2 == nullptr && a.g.slice_stride == 1 &&
         (a.g.ea % 2) == 0 && (a.g.eb % 2) == 0 && (reinterpret_cast<uintptr_t>(a.psi) % 16) == 0) {
-      pass_fast2d_pair_kernel<Real><<<(unsigned)((a.g.nslices + 1) / 2), 256, smem, st>>>(a);
+      pass_fast2d_pair_kernel<Real><<<(unsigned)((n + 1) / 2), 256, f2_smem<Real, MODE_STEP, false, 64, 1, false>(), st>>>(a);
       return cudaGetLastError();
     }
   }
-  if (a.mode == MODE_LAZY) pass_fast2d_kernel<Real, MODE_LAZY><<<(unsigned)ntiles, 256, smem, st>>>(a);
-  else if (a.T2) pass_fast2d_kernel<Real, MODE_STEP, true><<<(unsigned)ntiles, 256, smem, st>>>(a);
-  else pass_fast2d_kernel<Real, MODE_STEP><<<(unsigned)ntiles, 256, smem, st>>>(a);
+  if constexpr (N < 64) {
+    if (a.mode == MODE_STEP && a.list == nullptr && a.T2 == nullptr && a.g.slice_stride == 1) {
+      LS_F2K(MODE_STEP, false, N, SS, true)<<<(unsigned)((n + SS - 1) / SS), SS * 4 * N,
+                                              f2_smem<Real, MODE_STEP, false, N, SS, true>(), st>>>(a);
+      return cudaGetLastError();
+    }
+  }
+  if (a.mode == MODE_LAZY)
+    LS_F2K(MODE_LAZY, false, N, SC, false)<<<bc, SC * 4 * N, f2_smem<Real, MODE_LAZY, false, N, SC, false>(), st>>>(a);
+  else if (a.T2)
+    LS_F2K(MODE_STEP, true, N, SC, false)<<<bc, SC * 4 * N, f2_smem<Real, MODE_STEP, true, N, SC, false>(), st>>>(a);
+  else
+    LS_F2K(MODE_STEP, false, N, SC, false)<<<bc, SC * 4 * N, f2_smem<Real, MODE_STEP, false, N, SC, false>(), st>>>(a);
   return cudaGetLastError();
 }
 
-template <typename Real> cudaError_t fast2d_prepare(size_t max_smem) {
-  cudaError_t e = allow_smem(pass_fast2d_kernel<Real, MODE_STEP>, max_smem);
-  if (e == cudaSuccess) e = allow_smem(pass_fast2d_kernel<Real, MODE_STEP, true>, max_smem);
-  if constexpr (sizeof(Real) == 4)
-    if (e == cudaSuccess) e = allow_smem(pass_fast2d_pair_kernel<Real>, max_smem);
-  if (e == cudaSuccess) e = allow_smem(pass_fast2d_kernel<Real, MODE_LAZY>, max_smem);
+template <typename Real> cudaError_t launch_fast2d(const PassArgs& a, int64_t nslices, cudaStream_t st) {
+  if (nslices <= 0) return cudaSuccess;
+  if (a.g.d != 2 || a.g.qa != a.g.qb) return cudaErrorInvalidValue;
+  switch (a.g.qa) {
+    case 16: return launch_fast2d_n<Real, 16>(a, nslices, st);
+    case 32: return launch_fast2d_n<Real, 32>(a, nslices, st);
+    case 64: return launch_fast2d_n<Real, 64>(a, nslices, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <typename Real, int N> static cudaError_t fast2d_prepare_n(size_t max_smem) {
+  constexpr int SC = F2Slices<N>::kC, SS = F2Slices<N>::kS;
+  cudaError_t e = allow_smem(LS_F2K(MODE_STEP, false, N, SC, false), max_smem);
+  if (e == cudaSuccess) e = allow_smem(LS_F2K(MODE_STEP, true, N, SC, false), max_smem);
+  if (e == cudaSuccess) e = allow_smem(LS_F2K(MODE_LAZY, false, N, SC, false), max_smem);
+  if constexpr (N < 64)
+    if (e == cudaSuccess) e = allow_smem(LS_F2K(MODE_STEP, false, N, SS, true), max_smem);
   return e;
 }
+template <typename Real> cudaError_t fast2d_prepare(size_t max_smem) {
+  cudaError_t e = fast2d_prepare_n<Real, 64>(max_smem);
+  if (e == cudaSuccess) e = fast2d_prepare_n<Real, 32>(max_smem);
+  if (e == cudaSuccess) e = fast2d_prepare_n<Real, 16>(max_smem);
+  if constexpr (sizeof(Real) == 4)
+    if (e == cudaSuccess) e = allow_smem(pass_fast2d_pair_kernel<Real>, max_smem);
+  return e;
+}
+#undef LS_F2K
 
 // Two adjacent columns per CTA for the strided 1D layer (slice stride 1
 // element, transform length 4096, complex64): one 16-byte load or store moves
