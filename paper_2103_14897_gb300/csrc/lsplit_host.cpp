@@ -214,6 +214,7 @@ struct ls_ctx {
   int mask_mode = LS_MASK_INIT_ONLY;
   DevBuf maskbuf;   // joint-cutoff mask (M2 x M1 bytes), built on the first projecting step
   DevBuf partials, result, touch_row, touch_col, seedbuf, grad[2];
+  DevBuf densbuf;   // workspace of ls_density (allocated on first use)
   DevBuf scratch;   // second state array of the out-of-place semi-implicit step (allocated on first use)
   int nblk_elem = 0;
   size_t partial_count = 0;
@@ -354,7 +355,11 @@ std::vector<cd> conv_kernel(const ls_ctx* c, int layer, double s) {
   }
   for (int j = 0; j < q; ++j) {
     cd acc(0, 0);
-    for (int p2 = 0; p2 < q; ++p2) acc += tm1[p2] * roots[(int)(((int64_t)j * p2) % q)];
+    for (int p2 = 0, r = 0; p2 < q; ++p2) {   // r = j p2 mod q
+      acc += tm1[p2] * roots[r];
+      r += j;
+      if (r >= q) r -= q;
+    }
     cp[j] = acc / (double)q;
   }
   return cp;
@@ -668,6 +673,10 @@ void choose_launch(ls_ctx* c) {
                    : std::max(1, std::min(lsk::kMaxTileSlices, 8192 / g.buf));
     if (L == 1 && W < 2 && g.nslices > 1) W = 2;
     if ((int64_t)W > g.nslices) W = (int)g.nslices;
+    // small boxes: narrower tiles, so that about two CTAs share an SM (an
+    // adjoint pass of 513 x 513 ran on 129 and 65 CTAs: 84 and 125 us, 79 and
+    // 75 us so)
+    while (W > (L == 0 ? 1 : 2) && (g.nslices + W - 1) / W < 2 * (int64_t)c->sms) W = (W + 1) / 2;
     int bpt = 2, nt = 0;
     for (;;) {
       nt = lsk::pass_threads(g, W, 2);
@@ -795,10 +804,19 @@ cudaError_t launch(ls_ctx* c, const lsk::PassArgs& a0, int L, int64_t nitems, cu
     if (c->dtype == LS_C64) return lsk::launch_fast<float>(a, ntiles, st);
     return lsk::launch_fast<double>(a, ntiles, st);
   }
-  const lsk::PassArgs& a = a0;
+  lsk::PassArgs a = a0;
   const int64_t ntiles = (nitems + a.W - 1) / a.W;
-  if (c->dtype == LS_C64) return lsk::launch_pass<float>(a, c->bpt[L], c->nt[L], ntiles, st);
-  return lsk::launch_pass<double>(a, c->bpt[L], c->nt[L], ntiles, st);
+  int nt = c->nt[L];
+  if (a.mode == lsk::MODE_ADJOINT) {
+    // psi and lambda through the transform stages together where a CTA has the
+    // threads for twice the slices (513 x 513: 79 and 75 -> 55 and 59 us per factor)
+    const int nt2 = lsk::pass_threads(c->geom[L], 2 * a.W, c->bpt[L]);
+    const int most = c->dtype == LS_C64 ? lsk::pass_max_threads<float>(c->bpt[L]) : lsk::pass_max_threads<double>(c->bpt[L]);
+    a.variant = nt2 <= most;
+    if (a.variant) nt = std::max(nt, nt2);
+  }
+  if (c->dtype == LS_C64) return lsk::launch_pass<float>(a, c->bpt[L], nt, ntiles, st);
+  return lsk::launch_pass<double>(a, c->bpt[L], nt, ntiles, st);
 }
 
 int base_scheme(int scheme) {
@@ -1564,6 +1582,7 @@ int ls_create(const ls_problem* prob, ls_ctx** out) {
     c->M2 = (int64_t)prob->q2[0] * (prob->d > 1 ? prob->q2[1] : 1);
     c->pitch = (c->M1 + 15) / 16 * 16;
     LS_CUDA(cudaGetDevice(&c->device));
+    LS_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
     build_geometry(c.get());
     if (c->dtype == LS_C64) choose_launch<float>(c.get());
     else choose_launch<double>(c.get());
@@ -1627,7 +1646,6 @@ int ls_create(const ls_problem* prob, ls_ctx** out) {
     if (c->dtype == LS_C64) LS_CUDA(lsk::stencil_prepare<float>(block_max));
     else LS_CUDA(lsk::stencil_prepare<double>(block_max));
     for (int L = 0; L < 2; ++L) c->stW[L] = stencil_width(c->geom[L], c->esize, L == 1);
-    LS_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
     // tensor-core form of the contiguous 64 x 64 layer (complex64)
     if (c->dtype == LS_C64 && c->d == 2 && !c->p.shared && c->geom[0].qa == 64 && c->geom[0].qb == 64 &&
         lsk::tc2d_smem_bytes() + 8192 <= (size_t)dev_max + static_reserve && getenv_flag("LSPLIT_TC2D")) {
@@ -1907,12 +1925,20 @@ int ls_density(ls_ctx* c, const void* psi, const double* x, int64_t nx, double* 
     // (chunk * (M1 + 2 M2) complex elements) stay below 512 MB
     const int64_t per_point = (c->M1 + 2 * c->M2) * (int64_t)c->esize;
     const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nx, ((int64_t)512 << 20) / per_point));
-    DevBuf fb, e1, e2, t, ob;
-    fb.alloc((size_t)4 * chunk * sizeof(uint64_t));
-    e1.alloc((size_t)chunk * c->M1 * c->esize);
-    e2.alloc((size_t)chunk * c->M2 * c->esize);
-    t.alloc((size_t)chunk * c->M2 * c->esize);
-    ob.alloc((size_t)2 * nx * sizeof(double));
+    // one workspace, kept by the context up to 256 MB (allocating and freeing
+    // five buffers took 0.6 ms of a 3.2 ms call)
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t b_f = up((size_t)4 * chunk * sizeof(uint64_t)), b_1 = up((size_t)chunk * c->M1 * c->esize),
+                 b_2 = up((size_t)chunk * c->M2 * c->esize), b_o = up((size_t)2 * nx * sizeof(double));
+    const size_t need = b_f + b_1 + 2 * b_2 + b_o;
+    DevBuf once;
+    DevBuf& ws = need <= ((size_t)256 << 20) ? c->densbuf : once;
+    if (ws.bytes < need) ws.alloc(need);
+    struct View {
+      void* p;
+    };
+    char* wp = static_cast<char*>(ws.p);
+    const View fb{wp}, e1{wp + b_f}, e2{wp + b_f + b_1}, t{wp + b_f + b_1 + b_2}, ob{wp + b_f + b_1 + 2 * b_2};
     std::vector<uint64_t> f((size_t)4 * chunk, 0);
     for (int64_t j0 = 0; j0 < nx; j0 += chunk) {
       const int64_t cn = std::min(chunk, nx - j0);

@@ -566,12 +566,16 @@ __device__ __forceinline__ void pass_tile(const PassArgs& a, int64_t tile, unsig
   __syncthreads();
 
   // ---- to layer j's real-space grid (unnormalised inverse transform)
+  // (adjoint: lambda's slices follow psi's in shared memory; with the threads
+  // for both, a.variant 1, they go through the stages together)
+  const bool both = adj && a.variant == 1;
+  const int WT = both ? 2 * W : W;
   if (g.bluestein) {
-    bluestein_conv<Real, BPT>(sm, g, W, (const C*)g.bm);
-    if (adj) bluestein_conv<Real, BPT>(sml, g, W, (const C*)g.bm);
+    bluestein_conv<Real, BPT>(sm, g, WT, (const C*)g.bm);
+    if (adj && !both) bluestein_conv<Real, BPT>(sml, g, W, (const C*)g.bm);
   } else {
-    transform<Real, true, BPT, D1>(sm, g, W, false);
-    if (adj) transform<Real, true, BPT, D1>(sml, g, W, false);
+    transform<Real, true, BPT, D1>(sm, g, WT, false);
+    if (adj && !both) transform<Real, true, BPT, D1>(sml, g, W, false);
   }
 
   // ---- pointwise: (T - 1)/M, or the measurement / gradient
@@ -619,11 +623,11 @@ __device__ __forceinline__ void pass_tile(const PassArgs& a, int64_t tile, unsig
 
     // ---- back to coefficients (forward transform; 1/M is in the table)
     if (g.bluestein) {
-      bluestein_conv<Real, BPT>(sm, g, W, (const C*)g.bp);
-      if (adj) bluestein_conv<Real, BPT>(sml, g, W, (const C*)g.bp);
+      bluestein_conv<Real, BPT>(sm, g, WT, (const C*)g.bp);
+      if (adj && !both) bluestein_conv<Real, BPT>(sml, g, W, (const C*)g.bp);
     } else {
-      transform<Real, false, BPT, D1>(sm, g, W, false);
-      if (adj) transform<Real, false, BPT, D1>(sml, g, W, false);
+      transform<Real, false, BPT, D1>(sm, g, WT, false);
+      if (adj && !both) transform<Real, false, BPT, D1>(sml, g, W, false);
     }
 
     // ---- x + correction, kinetic post-phase, store
