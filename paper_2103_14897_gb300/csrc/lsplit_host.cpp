@@ -1646,6 +1646,25 @@ int ls_create(const ls_problem* prob, ls_ctx** out) {
     if (c->dtype == LS_C64) LS_CUDA(lsk::stencil_prepare<float>(block_max));
     else LS_CUDA(lsk::stencil_prepare<double>(block_max));
     for (int L = 0; L < 2; ++L) c->stW[L] = stencil_width(c->geom[L], c->esize, L == 1);
+    {
+      // rows: the width with the shortest time, waves of CTAs (three per SM) times
+      // the rows of a tile and about 1.5 rows' worth of tile overhead.  The widest
+      // tile leaves SMs idle on middle boxes and a nearly empty last wave on large
+      // ones: Strang, 20 steps, us, widest and chosen: 761 x 761 338 (10 rows) and
+      // 266 (3), 801 x 1801 542 (10) and 442 (4), 2049 x 2049 956 (4) and 945 (3).
+      // Columns keep the widest (761 x 761: 338 with 8, 346 with 4).
+      const int widest = c->stW[0];
+      const int64_t slots = 3 * (int64_t)c->sms, S = c->geom[0].nslices;
+      double least = 0;
+      for (int w = widest; w >= std::min(widest, 2); --w) {
+        const int64_t tiles = (S + w - 1) / w;
+        const double cost = (double)((tiles + slots - 1) / slots) * (w + 1.5);
+        if (w == widest || cost < least) {
+          least = cost;
+          c->stW[0] = w;
+        }
+      }
+    }
     // tensor-core form of the contiguous 64 x 64 layer (complex64)
     if (c->dtype == LS_C64 && c->d == 2 && !c->p.shared && c->geom[0].qa == 64 && c->geom[0].qb == 64 &&
         lsk::tc2d_smem_bytes() + 8192 <= (size_t)dev_max + static_reserve && getenv_flag("LSPLIT_TC2D")) {
