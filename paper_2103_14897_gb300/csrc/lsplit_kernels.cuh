@@ -1099,13 +1099,14 @@ pass_fast_kernel(const PassArgs a) {
 // elements j + 4k (k < N/4), two Stockham stages (radix 8 x 8, 8 x 4, 4 x 4)
 // exchange within the line, so inside a transform only the warp synchronises;
 // the CTA does between the axes, three times per factor.  32 x 32 slices (the
-// 32^4 box, 10 Strang steps) took 1116 us on the general pass and take 312 us;
-// 64 x 64 slices take 16 % fewer instructions than with a quarter of the line
-// per warp and thirteen barriers, and the same time (MIO and FMA queues).
+// 32^4 box, 10 Strang steps) took 1116 us on the general pass and take 312 us.
 // A half warp covers four lines; stride N + 4 = 4 modulo 16 puts its accesses
 // on distinct banks along both axes.
+// 64 x 64 keeps a quarter of the line per warp (lanes on 32 consecutive lines,
+// row stride 65): with quads it took fewer instructions, but 64^4 2297 us
+// against 2289 us.
 template <int N> struct F2 {
-  static constexpr int kRow = N + 4, kE = N / 4, kThreads = 4 * N;
+  static constexpr int kRow = N == 64 ? 65 : N + 4, kE = N / 4, kThreads = 4 * N;
   static constexpr int kR1 = N == 16 ? 4 : 8, kR2 = N / kR1;
 };
 
@@ -1150,6 +1151,36 @@ __device__ __forceinline__ void fft_quad(typename CT<Real>::C (&v)[N / 4], typen
     for (int r = 0; r < R2; ++r) v[u + U2 * r] = z[u * R2 + r];
   }
 }
+// 64 points, the CTA synchronising: thread j = 0..3 of a line holds elements
+// j + 4u + 8r (u < 2, r < 8) in v[8u + r]; two radix-8 stages.
+template <typename Real, bool INV>
+__device__ __forceinline__ void fft64_line(typename CT<Real>::C (&v)[16], typename CT<Real>::C* buf, int base,
+                                           int es, int j, const typename CT<Real>::C* __restrict__ tw) {
+  using C = typename CT<Real>::C;
+  C wb[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) wb[u] = tw[j + 4 * u];  // W_64^b, b = j + 4u (stage 2, stride 1)
+  // stage 1 (ns = 1): butterfly b = j + 4u reads x[b + 8r], writes 8b + r
+#pragma unroll
+  for (int u = 0; u < 2; ++u) dftR<8, C, INV>(v + 8 * u);
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int r = 0; r < 8; ++r) buf[base + (8 * (j + 4 * u) + r) * es] = v[8 * u + r];
+  __syncthreads();
+  // stage 2 (ns = 8): butterfly b reads x[b + 8r], twiddles W_64^(r b), writes b + 8r
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[8 * u + r] = buf[base + (j + 4 * u + 8 * r) * es];
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    twiddle_pow<8, Real, INV>(v + 8 * u, wb[u]);
+    dftR<8, C, INV>(v + 8 * u);
+  }
+}
+
 template <typename C, int E> __device__ __forceinline__ void quad_load(C (&v)[E], const C* buf, int base, int es, int j) {
 #pragma unroll
   for (int k = 0; k < E; ++k) v[k] = buf[base + (j + 4 * k) * es];
@@ -1184,7 +1215,8 @@ struct QuadWalk {
 
 // The correction F diag((T - 1)/M) F^{-1} x of one slice held in buf, in
 // place: inverse transforms along a and b, the potential factor, forward
-// transforms along b and a.  Thread r of the slice's 4 N takes line r / 4.
+// transforms along b and a.  Thread r of the slice's 4 N takes line r / 4
+// (64: line r mod 64).
 // Called after a CTA barrier, ends with one.
 template <typename Real, int N>
 __device__ __forceinline__ void f2_correction(typename CT<Real>::C* buf, const typename CT<Real>::C* __restrict__ T,
@@ -1192,26 +1224,63 @@ __device__ __forceinline__ void f2_correction(typename CT<Real>::C* buf, const t
                                               const typename CT<Real>::C* __restrict__ twb, int r) {
   using C = typename CT<Real>::C;
   constexpr int E = N / 4, RS = F2<N>::kRow;
-  const int sub = r >> 2, j = r & 3;
   C v[E];
-  // inverse transform along a (line = row ib = sub)
-  quad_load(v, buf, sub * RS, 1, j);
-  fft_quad<Real, true, N>(v, buf, sub * RS, 1, j, twa);
-  quad_store(v, buf, sub * RS, 1, j);
-  __syncthreads();
-  // inverse along b (line = column ia = sub), potential factor, forward along b
-  quad_load(v, buf, sub, RS, j);
-  fft_quad<Real, true, N>(v, buf, sub, RS, j, twb);
+  if constexpr (N == 64) {
+    const int sub = r & 63, j = r >> 6;
+    // v[8u + r] holds element j + 4u + 8r
+    auto load = [&](int base, int es) {
 #pragma unroll
-  for (int k = 0; k < E; ++k) v[k] = cmul(v[k], T[sub + N * (j + 4 * k)]);
-  fft_quad<Real, false, N>(v, buf, sub, RS, j, twb);
-  quad_store(v, buf, sub, RS, j);
-  __syncthreads();
-  // forward along a
-  quad_load(v, buf, sub * RS, 1, j);
-  fft_quad<Real, false, N>(v, buf, sub * RS, 1, j, twa);
-  quad_store(v, buf, sub * RS, 1, j);
-  __syncthreads();
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[8 * u + q] = buf[base + (j + 4 * u + 8 * q) * es];
+    };
+    auto store = [&](int base, int es) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) buf[base + (j + 4 * u + 8 * q) * es] = v[8 * u + q];
+    };
+    load(sub * RS, 1);
+    __syncthreads();
+    fft64_line<Real, true>(v, buf, sub * RS, 1, j, twa);
+    store(sub * RS, 1);
+    __syncthreads();
+    load(sub, RS);
+    __syncthreads();
+    fft64_line<Real, true>(v, buf, sub, RS, j, twb);
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[8 * u + q] = cmul(v[8 * u + q], T[sub + 64 * (j + 4 * u + 8 * q)]);
+    fft64_line<Real, false>(v, buf, sub, RS, j, twb);
+    store(sub, RS);
+    __syncthreads();
+    load(sub * RS, 1);
+    __syncthreads();
+    fft64_line<Real, false>(v, buf, sub * RS, 1, j, twa);
+    store(sub * RS, 1);
+    __syncthreads();
+  } else {
+    const int sub = r >> 2, j = r & 3;
+    // inverse transform along a (line = row ib = sub)
+    quad_load(v, buf, sub * RS, 1, j);
+    fft_quad<Real, true, N>(v, buf, sub * RS, 1, j, twa);
+    quad_store(v, buf, sub * RS, 1, j);
+    __syncthreads();
+    // inverse along b (line = column ia = sub), potential factor, forward along b
+    quad_load(v, buf, sub, RS, j);
+    fft_quad<Real, true, N>(v, buf, sub, RS, j, twb);
+  #pragma unroll
+    for (int k = 0; k < E; ++k) v[k] = cmul(v[k], T[sub + N * (j + 4 * k)]);
+    fft_quad<Real, false, N>(v, buf, sub, RS, j, twb);
+    quad_store(v, buf, sub, RS, j);
+    __syncthreads();
+    // forward along a
+    quad_load(v, buf, sub * RS, 1, j);
+    fft_quad<Real, false, N>(v, buf, sub * RS, 1, j, twa);
+    quad_store(v, buf, sub * RS, 1, j);
+    __syncthreads();
+  }
 }
 
 // SP slices per CTA of SP 4 N threads.  For loads and stores thread t takes
