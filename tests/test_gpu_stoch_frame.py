@@ -88,3 +88,22 @@ def test_sampler(P, n):
         got = ctx.samples(2, seed=77, g0=5, count=3)
         for r in range(3):
             assert np.array_equal(got[r], np.asarray(O.sample_slices(S, k, 77, 5 + r))), (S, frac_den, r)
+
+
+def test_batch_timeout_hook(P):
+    """The hook that makes a wait unsatisfiable still ends a stochastic call
+    with LS_ERR_TIMEOUT, and the batch works again afterwards."""
+    probs = W.batch_1d(count=3, seed=2, nmin=8, nmax=20)
+    b = P.Batch(probs, "c64")
+    psi = b.empty()
+    b.debug(True, 0.2)
+    with pytest.raises(P.LsplitError) as e:
+        b.step(psi, 2, 1e-3, "strang_stoch", seed=1)
+    assert e.value.code == P.LS_ERR_TIMEOUT
+    b.debug(False, 1.0)
+    xs = [W.random_state((p.M2, p.M1), 90 + i) for i, p in enumerate(probs)]
+    for i, x in enumerate(xs):
+        b.set_dense(psi, i, x)
+    b.step(psi, 2, 1e-3, "strang_stoch", seed=1)
+    for i, p in enumerate(probs):
+        assert rel(b.get_dense(psi, i), O.step(p, xs[i], 1e-3, "strang_stoch", 2, seed=1 + i)) < 3e-5
