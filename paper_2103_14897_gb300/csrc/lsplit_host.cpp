@@ -904,6 +904,35 @@ lsk::SamplerArgs sampler_args(ls_ctx* c, int scheme, int& npf) {
   return sa;
 }
 
+// |Lambda| of one step of a deterministic 1D scheme whose factors all take the
+// compact-kernel form: the factors' scalar parts 1 + c'_0, which the interaction
+// frame collects.  0: the frame is not available (another scheme, a factor in
+// another form, or a step that leaves less than 1/16).
+double frame_decay(ls_ctx* c, int scheme, double tau) {
+  if (c->d != 1 || (scheme != LS_LIE && scheme != LS_STRANG && scheme != LS_STRANG_KP)) return 0.0;
+  std::vector<PassSpec> ps;
+  int32_t end = 0;
+  build_passes(scheme, tau, 1, ps, end);
+  double d = 1.0;
+  for (const PassSpec& q : ps) {
+    const CachedTab t = stencil_table(c, q.layer, q.s);
+    if (t.B == 0) return 0.0;
+    d *= std::abs(t.diag);
+  }
+  return d >= 0.0625 ? d : 0.0;
+}
+
+// Steps that one interaction-frame graph may hold.  The frame's state grows as
+// 1 / |Lambda| and Lambda is applied as 1 - (1 - |Lambda|): beyond |Lambda| =
+// 1/2 that cancels (and overflows in FP32 later), so a longer call runs as
+// pieces, each ending with its own Lambda K(T).  (Without the limit a complex64
+// call of 2000 Strang steps with tau max|v| = 0.2 returned rounding noise.)
+int64_t frame_steps(double decay) {
+  if (decay <= 0.0 || decay >= 1.0) return INT64_MAX;
+  const double m = std::log(0.5) / std::log(decay);
+  return m >= 1e15 ? INT64_MAX : std::max<int64_t>(1, (int64_t)m);
+}
+
 // ---- tile form of a deterministic compact-kernel call (lsplit_tile.cu)
 
 // Taps of one layer for the tile form: its half-width class (0: the layer does
@@ -977,6 +1006,7 @@ int tile_instance(ls_ctx* c, int scheme, double tau, int64_t n, lsk::TileInst* i
   // us: 33 x 33 100 against 191, 257 x 257 121 / 328, 513 x 513 205 / 350),
   // beyond the halos cost more than the launches (769 x 769 381 / 343).
   if (c->dtype == LS_C64 && c->M1 * c->M2 > (int64_t)c->sms * 4 * 24 * 28) return 0;
+  if (frame_decay(c, scheme, tau) == 0.0) return 0;
   lsk::TileInst in;
   std::memset(&in, 0, sizeof(in));
   int bv = 0;
@@ -1342,7 +1372,8 @@ void enqueue_step(ls_ctx* c, void* psi, int64_t n, double tau, int scheme, cudaS
   // factors' scalar parts).
   bool ip = !stoch && c->d == 1 && c->dtype == LS_C64 &&
             (scheme == LS_LIE || scheme == LS_STRANG || scheme == LS_STRANG_KP) && !getenv_flag("LSPLIT_NO_IP");
-  for (size_t i = 0; i < ps.size() && ip; ++i) ip = !ps[i].fused && stencil_table(c, ps[i].layer, ps[i].s).B > 0;
+  ip = ip && frame_decay(c, scheme, tau) > 0.0;
+  for (size_t i = 0; i < ps.size() && ip; ++i) ip = !ps[i].fused;
   int64_t t_acc = 0;
   std::complex<double> lam(1.0, 0.0);
   for (size_t i = 0; i < ps.size(); ++i) {
@@ -1464,6 +1495,82 @@ void prepare_tables(ls_ctx* c, int64_t n, double tau, int scheme) {
     phase_table(c, q.layer, sd);
     if (stencil_table(c, q.layer, sd).B == 0 && c->conv_form[q.layer - 1]) conv_table(c, q.layer, sd);
   }
+}
+
+// The cached graph of a call, moved to the front of the list; NULL if there is none.
+GraphEntry* find_graph(ls_ctx* c, void* psi, int64_t n, double tau, int scheme) {
+  for (auto it = c->graphs.begin(); it != c->graphs.end(); ++it) {
+    GraphEntry* e = it->get();
+    if (e->psi == psi && e->scheme == scheme && e->tau == tau && e->n == n) {
+      c->graphs.splice(c->graphs.begin(), c->graphs, it);
+      return e;
+    }
+  }
+  return nullptr;
+}
+
+// Capture n steps on psi and keep the graph (at most 8 per context).
+GraphEntry* build_graph(ls_ctx* c, void* psi, int64_t n, double tau, int scheme) {
+  const bool stoch = scheme == LS_LIE_STOCH || scheme == LS_STRANG_STOCH || scheme == LS_RANDOM_BATCH;
+  std::unique_ptr<GraphEntry> e(new GraphEntry());
+  e->psi = psi;
+  e->scheme = scheme;
+  e->tau = tau;
+  e->n = n;
+  e->lists = std::make_shared<DevBuf>();
+  if (stoch) {
+    int npf = 0;
+    lsk::SamplerArgs sa = sampler_args(c, scheme, npf);
+    e->lists->alloc((size_t)n * npf * sa.pmax * sizeof(int32_t));
+  }
+  if (c->mask_mode == LS_MASK_PROJECT_EACH_STEP && !c->maskbuf.p) {
+    std::vector<uint8_t> m((size_t)(c->M1 * c->M2));
+    joint_mask(c, m.data());
+    c->maskbuf.alloc(m.size());
+    LS_CUDA(cudaMemcpy(c->maskbuf.p, m.data(), m.size(), cudaMemcpyHostToDevice));
+  }
+  // Tables are built (and uploaded) before capture: no allocation or
+  // synchronous copy may happen while the stream is being captured.  The
+  // graph keeps a reference to every table it reads.
+  struct KeepScope {
+    ls_ctx* c;
+    ~KeepScope() { c->keep = nullptr; }
+  } ks{c};
+  c->keep = &e->tables;
+  if ((reinterpret_cast<uintptr_t>(psi) & 15) == 0 && tile_instance(c, scheme, tau, n, nullptr)) {
+    tile_tables(c);
+    // the second state array, one per psi (graphs of other arrays may run
+    // on other streams); without room for it the call runs in place
+    for (auto& g : c->graphs)
+      if (g->psi == psi && g->alt) e->alt = g->alt;
+    if (!e->alt) {
+      try {
+        e->alt = std::make_shared<DevBuf>();
+        e->alt->alloc((size_t)c->pitch * c->M2 * c->esize);
+      } catch (const CudaError& ce) {
+        e->alt.reset();
+        cudaGetLastError();
+        if (ce.e != cudaErrorMemoryAllocation) throw;
+      }
+    }
+  }
+  if (!e->alt) prepare_tables(c, n, tau, scheme);
+  cudaGraph_t graph = nullptr;
+  LS_CUDA(cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal));
+  try {
+    enqueue_step(c, psi, n, tau, scheme, c->cap, e->lists.get(), e->alt ? e->alt->p : nullptr);
+  } catch (...) {
+    cudaStreamEndCapture(c->cap, &graph);
+    if (graph) cudaGraphDestroy(graph);
+    throw;
+  }
+  LS_CUDA(cudaStreamEndCapture(c->cap, &graph));
+  cudaError_t ie = cudaGraphInstantiate(&e->exec, graph, 0);
+  cudaGraphDestroy(graph);
+  if (ie != cudaSuccess) throw CudaError{ie, "cudaGraphInstantiate"};
+  c->graphs.push_front(std::move(e));
+  while (c->graphs.size() > 8) c->graphs.pop_back();
+  return c->graphs.front().get();
 }
 
 template <typename F>
@@ -1800,77 +1907,22 @@ int ls_step(ls_ctx* c, void* psi, int64_t n, double tau, int32_t scheme, uint64_
       // pageable source: staged before the call returns, safe to reuse
       LS_CUDA(cudaMemcpyAsync(c->seedbuf.p, hp, sizeof(hp), cudaMemcpyHostToDevice, st));
     }
-    GraphEntry* ge = nullptr;
-    for (auto it = c->graphs.begin(); it != c->graphs.end(); ++it) {
-      GraphEntry* e = it->get();
-      if (e->psi == psi && e->scheme == scheme && e->tau == tau && e->n == n) {
-        ge = e;
-        c->graphs.splice(c->graphs.begin(), c->graphs, it);
-        break;
-      }
+    if (GraphEntry* ge = find_graph(c, psi, n, tau, scheme)) {
+      LS_CUDA(cudaGraphLaunch(ge->exec, st));
+      return LS_OK;
     }
-    if (!ge) {
-      std::unique_ptr<GraphEntry> e(new GraphEntry());
-      e->psi = psi;
-      e->scheme = scheme;
-      e->tau = tau;
-      e->n = n;
-      e->lists = std::make_shared<DevBuf>();
-      if (stoch) {
-        int npf = 0;
-        lsk::SamplerArgs sa = sampler_args(c, scheme, npf);
-        e->lists->alloc((size_t)n * npf * sa.pmax * sizeof(int32_t));
-      }
-      if (c->mask_mode == LS_MASK_PROJECT_EACH_STEP && !c->maskbuf.p) {
-        std::vector<uint8_t> m((size_t)(c->M1 * c->M2));
-        joint_mask(c, m.data());
-        c->maskbuf.alloc(m.size());
-        LS_CUDA(cudaMemcpy(c->maskbuf.p, m.data(), m.size(), cudaMemcpyHostToDevice));
-      }
-      // Tables are built (and uploaded) before capture: no allocation or
-      // synchronous copy may happen while the stream is being captured.  The
-      // graph keeps a reference to every table it reads.
-      struct KeepScope {
-        ls_ctx* c;
-        ~KeepScope() { c->keep = nullptr; }
-      } ks{c};
-      c->keep = &e->tables;
-      if ((reinterpret_cast<uintptr_t>(psi) & 15) == 0 && tile_instance(c, scheme, tau, n, nullptr)) {
-        tile_tables(c);
-        // the second state array, one per psi (graphs of other arrays may run
-        // on other streams); without room for it the call runs in place
-        for (auto& g : c->graphs)
-          if (g->psi == psi && g->alt) e->alt = g->alt;
-        if (!e->alt) {
-          try {
-            e->alt = std::make_shared<DevBuf>();
-            e->alt->alloc((size_t)c->pitch * c->M2 * c->esize);
-          } catch (const CudaError& ce) {
-            e->alt.reset();
-            cudaGetLastError();
-            if (ce.e != cudaErrorMemoryAllocation) throw;
-          }
-        }
-      }
-      if (!e->alt) prepare_tables(c, n, tau, scheme);
-      cudaGraph_t graph = nullptr;
-      LS_CUDA(cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal));
-      try {
-        enqueue_step(c, psi, n, tau, scheme, c->cap, e->lists.get(), e->alt ? e->alt->p : nullptr);
-      } catch (...) {
-        cudaStreamEndCapture(c->cap, &graph);
-        if (graph) cudaGraphDestroy(graph);
-        throw;
-      }
-      LS_CUDA(cudaStreamEndCapture(c->cap, &graph));
-      cudaError_t ie = cudaGraphInstantiate(&e->exec, graph, 0);
-      cudaGraphDestroy(graph);
-      if (ie != cudaSuccess) throw CudaError{ie, "cudaGraphInstantiate"};
-      c->graphs.push_front(std::move(e));
-      while (c->graphs.size() > 8) c->graphs.pop_back();
-      ge = c->graphs.front().get();
-    }
-    LS_CUDA(cudaGraphLaunch(ge->exec, st));
+    // a call that decays too far for one interaction-frame graph runs as pieces
+    // (both graphs exist before the first of them runs)
+    const bool frame = c->dtype == LS_C64 ? !getenv_flag("LSPLIT_NO_IP") : tile_instance(c, scheme, tau, 1, nullptr) > 0;
+    const int64_t piece = frame ? std::min(n, frame_steps(frame_decay(c, scheme, tau))) : n;
+    auto graph = [&](int64_t m) {
+      GraphEntry* ge = find_graph(c, psi, m, tau, scheme);
+      return ge ? ge : build_graph(c, psi, m, tau, scheme);
+    };
+    GraphEntry* rest = n % piece ? graph(n % piece) : nullptr;
+    GraphEntry* ge = graph(piece);
+    for (int64_t k = 0; k < n / piece; ++k) LS_CUDA(cudaGraphLaunch(ge->exec, st));
+    if (rest) LS_CUDA(cudaGraphLaunch(rest->exec, st));
     return LS_OK;
   });
 }
@@ -2293,6 +2345,9 @@ std::unique_ptr<ls_batch::Cached> build_batch_graph(ls_batch* b, void* psi, int6
                                   : ps[q].s;
         all_compact = b->Si1[L][i] > 0 && stencil_table(c, ps[q].layer, sdur).B > 0;
       }
+    // (that kernel's deterministic complex64 tiles are in the interaction frame)
+    for (int i = 0; i < ninst && all_compact && !stoch && b->dtype == LS_C64; ++i)
+      all_compact = frame_decay(b->inst[i], scheme, tau) > 0.0;
     const int kind = all_compact ? 1 : 0;
     // deterministic complex64 calls of the compact-only kernel run in the
     // interaction frame (kinetic factors folded into the taps, applied once at
@@ -2603,7 +2658,17 @@ bool batch_all_compact(ls_batch* b, double tau, int32_t scheme) {
       const double sd = stoch ? q.s * (double)S / (double)p : q.s;
       if (b->Si1[L][i] <= 0 || stencil_table(c, q.layer, sd).B == 0) return false;
     }
+  for (ls_ctx* c : b->inst)
+    if (!stoch && b->dtype == LS_C64 && frame_decay(c, scheme, tau) == 0.0) return false;
   return true;
+}
+
+// Steps per graph of a deterministic complex64 call: the least of the
+// instances' frame_steps.
+int64_t batch_piece(ls_batch* b, double tau, int32_t scheme, int64_t n) {
+  if (b->dtype != LS_C64 || !batch_all_compact(b, tau, scheme)) return n;
+  for (ls_ctx* c : b->inst) n = std::min(n, frame_steps(frame_decay(c, scheme, tau)));
+  return n;
 }
 
 // Process-wide record of tuned configurations, keyed by the batch's shapes,
@@ -2930,18 +2995,28 @@ int ls_batch_step(ls_batch* b, void* psi, int64_t n, double tau, int32_t scheme,
       const uint64_t hp[2] = {seed, step0 * (uint64_t)factors_per_step(scheme)};
       LS_CUDA(cudaMemcpyAsync(b->seedbuf.p, hp, sizeof(hp), cudaMemcpyHostToDevice, st));
     }
-    ls_batch::Cached* ge = nullptr;
-    for (auto& e : b->graphs)
-      if (e->psi == psi && e->scheme == scheme && e->tau == tau && e->n == n) ge = e.get();
-    const int ninst = (int)b->inst.size();
-    if (!ge) {
-      maybe_tune(b, psi, n, tau, scheme, st);
-      std::unique_ptr<ls_batch::Cached> e = build_batch_graph(b, psi, n, tau, scheme);
-      b->graphs.push_front(std::move(e));
+    auto find = [&](int64_t m) -> ls_batch::Cached* {
+      for (auto& e : b->graphs)
+        if (e->psi == psi && e->scheme == scheme && e->tau == tau && e->n == m) return e.get();
+      return nullptr;
+    };
+    auto graph = [&](int64_t m) {
+      if (ls_batch::Cached* e = find(m)) return e;
+      b->graphs.push_front(build_batch_graph(b, psi, m, tau, scheme));
       while (b->graphs.size() > 4) b->graphs.pop_back();
-      ge = b->graphs.front().get();
+      return b->graphs.front().get();
+    };
+    if (ls_batch::Cached* ge = find(n)) {
+      LS_CUDA(cudaGraphLaunch(ge->exec, st));
+    } else {
+      maybe_tune(b, psi, n, tau, scheme, st);
+      // pieces as in ls_step
+      const int64_t piece = batch_piece(b, tau, scheme, n);
+      ls_batch::Cached* rest = n % piece ? graph(n % piece) : nullptr;
+      ge = graph(piece);
+      for (int64_t k = 0; k < n / piece; ++k) LS_CUDA(cudaGraphLaunch(ge->exec, st));
+      if (rest) LS_CUDA(cudaGraphLaunch(rest->exec, st));
     }
-    LS_CUDA(cudaGraphLaunch(ge->exec, st));
     int32_t status = 0;
     LS_CUDA(cudaMemcpyAsync(&status, b->status.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     LS_CUDA(cudaStreamSynchronize(st));

@@ -1,0 +1,65 @@
+"""Calls so long that the factors' scalar parts Lambda of the interaction frame
+decay far: one call against the same call cut into short ones.
+
+Tolerance: both round every factor; added up coherently over F factors that is
+at most F 2^-24 (complex64) and F 2^-53 (complex128) on each side."""
+import numpy as np
+import pytest
+
+import workloads as W
+from tests._parity import rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2103_14897_gb300 import build as B
+    B.build()
+    import paper_2103_14897_gb300 as P
+    P.load_library()
+    return P
+
+
+# |Lambda| of the whole call: 1e-13 and 1e-19 (complex64), 0.27 (complex128)
+@pytest.mark.parametrize("dtype,amp,tau,scheme,n,cuts", [
+    ("c64", 200.0, 1e-3, "strang", 2000, 100),
+    ("c64", 200.0, 1e-3, "lie", 2003, 100),
+    ("c64", 200.0, 1e-3, "strang_kp", 2000, 100),
+    ("c64", 50.0, 1e-3, "strang", 50000, 50),
+    ("c128", 3.4, 1e-3, "lie", 230000, 4),
+])
+@pytest.mark.parametrize("tiles", [True, False])
+def test_long_call_equals_its_pieces(P, monkeypatch, dtype, amp, tau, scheme, n, cuts, tiles):
+    if not tiles:
+        if dtype == "c128" or n > 10000:
+            pytest.skip("the in-place passes of complex128 are not in the frame; one long case is enough")
+        monkeypatch.setenv("LSPLIT_NO_TILE", "1")
+    p = W.bilayer_1d(13, 9, amp, 0.8 * amp, ecut=1e9)
+    ctx = P.Context(p, dtype)
+    x = W.random_state((p.M2, p.M1), 71)
+    one, cut = ctx.from_dense(x), ctx.from_dense(x)
+    ctx.step(one, n, tau, scheme)
+    for k in range(cuts):
+        ctx.step(cut, n // cuts + (n % cuts if k == 0 else 0), tau, scheme)
+    tol = 2 * 3 * n * (2.0 ** -24 if dtype == "c64" else 2.0 ** -53)
+    assert rel(ctx.to_dense(one), ctx.to_dense(cut)) < tol
+
+
+@pytest.mark.parametrize("scheme", ["strang", "lie"])
+def test_long_batched_call_equals_its_pieces(P, scheme):
+    probs = [W.bilayer_1d(13, 9, 200.0, 150.0, ecut=1e9), W.bilayer_1d(40, 20, 3.0, 2.0, ecut=1e9)]
+    b = P.Batch(probs, "c64")
+    xs = [W.random_state((p.M2, p.M1), 80 + i) for i, p in enumerate(probs)]
+    one, cut = b.empty(), b.empty()
+    for i, x in enumerate(xs):
+        b.set_dense(one, i, x)
+        b.set_dense(cut, i, x)
+    b.step(one, 2003, 1e-3, scheme)
+    for k in range(100):
+        b.step(cut, 20 + (3 if k == 0 else 0), 1e-3, scheme)
+    for i in range(2):
+        assert rel(b.get_dense(one, i), b.get_dense(cut, i)) < 2 * 3 * 2003 * 2.0 ** -24
