@@ -63,3 +63,20 @@ def test_long_batched_call_equals_its_pieces(P, scheme):
         b.step(cut, 20 + (3 if k == 0 else 0), 1e-3, scheme)
     for i in range(2):
         assert rel(b.get_dense(one, i), b.get_dense(cut, i)) < 2 * 3 * 2003 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("tiles", [True, False])
+@pytest.mark.parametrize("amp", [1.0, 2.4, 3.4])
+def test_long_complex128_call_keeps_the_norm(P, monkeypatch, tiles, amp):
+    """20000 Strang steps are unitary: the norm may move by the random roundings
+    of 60000 factors (60000^(1/2) 2^-53 = 3e-14) and by the factors' tables
+    (1e-18 each, 6e-14 if it all adds up); four times their sum."""
+    if not tiles:
+        monkeypatch.setenv("LSPLIT_NO_TILE", "1")
+    p = W.bilayer_1d(16, 12, amp, 0.8 * amp, ecut=1e9)
+    ctx = P.Context(p, "c128")
+    x = W.random_state((p.M2, p.M1), 72)
+    psi = ctx.from_dense(x)
+    ctx.step(psi, 20000, 1e-3, "strang")
+    got, want = np.linalg.norm(ctx.to_dense(psi)), np.linalg.norm(x)
+    assert abs(got / want - 1) < 4e-13
