@@ -223,7 +223,9 @@ int ls_observables(ls_ctx* ctx, const void* psi_dev, const void* chi_dev, ls_obs
  * point).  The phases are exact (64-bit fixed-point turns); the sum over m
  * runs in the context's precision, the sum over n in FP64.  The points are
  * processed in chunks whose temporary device buffers (chunk * (M1 + 2 M2)
- * complex elements) stay below 512 MB; synchronises the stream.
+ * complex elements) stay below 512 MB; the context keeps one such workspace of
+ * at most 256 MB between calls.  Several threads may call it on one context at
+ * once (each call has a workspace of its own).  Synchronises the stream.
  * LS_ERR_INVALID for nx beyond 2^22. */
 int ls_density(ls_ctx* ctx, const void* psi_dev, const double* x_host, int64_t nx, double* out_host,
                void* stream);

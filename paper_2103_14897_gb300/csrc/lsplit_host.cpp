@@ -223,7 +223,8 @@ struct ls_ctx {
   int mask_mode = LS_MASK_INIT_ONLY;
   DevBuf maskbuf;   // joint-cutoff mask (M2 x M1 bytes), built on the first projecting step
   DevBuf partials, result, touch_row, touch_col, seedbuf, grad[2];
-  DevBuf densbuf;   // workspace of ls_density (allocated on first use)
+  std::mutex dens_mu;
+  std::unique_ptr<DevBuf> densbuf;   // workspace between calls of ls_density (a call takes it out)
   DevBuf scratch;   // second state array of the out-of-place semi-implicit step (allocated on first use)
   int nblk_elem = 0;
   size_t partial_count = 0;
@@ -2006,18 +2007,24 @@ int ls_density(ls_ctx* c, const void* psi, const double* x, int64_t nx, double* 
     const int64_t per_point = (c->M1 + 2 * c->M2) * (int64_t)c->esize;
     const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nx, ((int64_t)512 << 20) / per_point));
     // one workspace, kept by the context up to 256 MB (allocating and freeing
-    // five buffers took 0.6 ms of a 3.2 ms call)
+    // five buffers took 0.6 ms of a 3.2 ms call).  A call owns it while it runs:
+    // calls of several threads or streams have one each, the larger is kept.
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t b_f = up((size_t)4 * chunk * sizeof(uint64_t)), b_1 = up((size_t)chunk * c->M1 * c->esize),
                  b_2 = up((size_t)chunk * c->M2 * c->esize), b_o = up((size_t)2 * nx * sizeof(double));
     const size_t need = b_f + b_1 + 2 * b_2 + b_o;
-    DevBuf once;
-    DevBuf& ws = need <= ((size_t)256 << 20) ? c->densbuf : once;
-    if (ws.bytes < need) ws.alloc(need);
+    constexpr size_t kKept = (size_t)256 << 20;
+    std::unique_ptr<DevBuf> ws;
+    if (need <= kKept) {
+      std::lock_guard<std::mutex> lk(c->dens_mu);
+      ws = std::move(c->densbuf);
+    }
+    if (!ws) ws.reset(new DevBuf());
+    if (ws->bytes < need) ws->alloc(need);
     struct View {
       void* p;
     };
-    char* wp = static_cast<char*>(ws.p);
+    char* wp = static_cast<char*>(ws->p);
     const View fb{wp}, e1{wp + b_f}, e2{wp + b_f + b_1}, t{wp + b_f + b_1 + b_2}, ob{wp + b_f + b_1 + 2 * b_2};
     std::vector<uint64_t> f((size_t)4 * chunk, 0);
     for (int64_t j0 = 0; j0 < nx; j0 += chunk) {
@@ -2062,6 +2069,10 @@ int ls_density(ls_ctx* c, const void* psi, const double* x, int64_t nx, double* 
     }
     LS_CUDA(cudaMemcpyAsync(out, ob.p, (size_t)2 * nx * sizeof(double), cudaMemcpyDeviceToHost, st));
     LS_CUDA(cudaStreamSynchronize(st));
+    if (ws->bytes <= kKept) {
+      std::lock_guard<std::mutex> lk(c->dens_mu);
+      if (!c->densbuf || c->densbuf->bytes < ws->bytes) std::swap(c->densbuf, ws);
+    }
     return LS_OK;
   });
 }
