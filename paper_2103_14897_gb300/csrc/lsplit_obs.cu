@@ -73,7 +73,29 @@ template <typename C> __device__ __forceinline__ void moments(Sum<double>* s, C 
 __device__ __forceinline__ uint32_t mag(float2 v) {
   return max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu);
 }
-constexpr uint32_t kLow = (127u - 48u) << 23, kHigh = (127u + 60u) << 23;   // 2^-48, 2^60
+// Components between which the sums of an item fit pairs of floats: up to 2^36
+// the second moment, at most 2 2^72 m'^2 per element and 16 elements per lane,
+// stays finite for |m'| < 2^24; from 2^-40 on what a product below 2^-102 loses
+// of its low part (2^-149 each, 2^11 of them) is 2^-58 of the item's norm.
+constexpr uint32_t kLow = (127u - 40u) << 23, kHigh = (127u + 36u) << 23;
+// Overlap products: below this the lost low parts would show (2^-138 of 2^-90)
+constexpr uint32_t kLowProd = (127u - 90u) << 23;
+
+// <chi, psi> over the elements [c0, c1) of a row
+template <typename Acc, typename C>
+__device__ __forceinline__ void overlap(const C* x, const C* y, int c0, int c1, double* ov) {
+  Acc re, im;
+#pragma unroll 4
+  for (int m = c0 + (threadIdx.x & 31); m < c1; m += 32) {
+    const C v = x[m], c = y[m];
+    re.mac(c.x, v.x);
+    re.mac(c.y, v.y);
+    im.mac(c.x, v.y);
+    im.mac(-c.y, v.x);
+  }
+  ov[0] = re.get();
+  ov[1] = im.get();
+}
 
 // One item: elements [c0, c1) of a row; Acc the accumulators' type.  Returns
 // false if a neighbour left the range of the pairs (nothing is added then).
@@ -96,18 +118,20 @@ __device__ __forceinline__ bool item(const ObsArgs& a, const C* psi, const C* ch
   uint32_t mx = 0;
   if (chi) {
     const C* y = chi + (int64_t)row * a.pitch;
-    Acc re, im;
+    uint32_t pm = 0, cm = 0;   // largest product and chi
+    if constexpr (pairs) {
 #pragma unroll 4
-    for (int m = c0 + lane; m < c1; m += 32) {
-      const C v = x[m], c = y[m];
-      if constexpr (pairs) mx = max(mx, mag(c));
-      re.mac(c.x, v.x);
-      re.mac(c.y, v.y);
-      im.mac(c.x, v.y);
-      im.mac(-c.y, v.x);
+      for (int m = c0 + lane; m < c1; m += 32) {
+        const uint32_t q = mag(y[m]);
+        cm = max(cm, q);
+        pm = max(pm, __float_as_uint(__fmul_rn(__uint_as_float(q), __uint_as_float(mag(x[m])))));
+      }
+      mx = cm;
+      pm = __reduce_max_sync(0xffffffffu, pm);
+      cm = __reduce_max_sync(0xffffffffu, cm);
     }
-    ov[0] = re.get();
-    ov[1] = im.get();
+    if (!pairs || (cm != 0 && pm < kLowProd)) overlap<Sum<double>>(x, y, c0, c1, ov);
+    else overlap<Acc>(x, y, c0, c1, ov);
   }
   // sum_m x_m conj(x_{m + h}) for the harmonics of both layers
 #pragma unroll 1
@@ -155,8 +179,8 @@ template <typename Real> __global__ void __launch_bounds__(256) obs1d_kernel(con
     const int row = (int)(it / nch), c0 = (int)(it - (int64_t)row * nch) * kObsChunk;
     const int c1 = min(a.M1, c0 + kObsChunk);
     if constexpr (sizeof(Real) == 4) {
-      // pairs of floats hold the products while the item's largest component
-      // is between 2^-48 and 2^60 (neighbours: below 2^60); else FP64
+      // pairs of floats while the item's largest component is between kLow and
+      // kHigh (chi and neighbours: below kHigh); else FP64
       uint32_t mx = 0;
 #pragma unroll 4
       for (int m = c0 + lane; m < c1; m += 32) mx = max(mx, mag(psi[(int64_t)row * a.pitch + m]));
