@@ -221,7 +221,9 @@ int ls_observables(ls_ctx* ctx, const void* psi_dev, const void* chi_dev, ls_obs
  *   psi(x_j) = sum_{m,n} phi[n][m] exp(i (B1 m + B2 n) . x_j),  j < nx.
  * x_host: nx points of d doubles each; out_host: 2 nx doubles (re, im per
  * point).  The phases are exact (64-bit fixed-point turns); the sum over m
- * runs in the context's precision, the sum over n in FP64.  The points are
+ * runs in the context's precision, the sum over n in FP64 (complex64: exact
+ * products added up in pairs of floats, 2^-48 per addition, 32 at a time, then
+ * in FP64).  The points are
  * processed in chunks whose temporary device buffers (chunk * (M1 + 2 M2)
  * complex elements) stay below 512 MB; the context keeps one such workspace of
  * at most 256 MB between calls.  Several threads may call it on one context at

@@ -7,7 +7,8 @@
 // of B^T x_j / 2 pi as 64-bit fractions per point; the integer index
 // components multiply them modulo 2^64), the contraction over m is a tiled
 // complex product (64 x 64 outputs per CTA, 16-wide slabs of m in shared
-// memory), the sum over n is one warp per point with FP64 accumulation.
+// memory), the sum over n is one warp per point, in FP64 (complex64: pairs of
+// floats, then FP64).
 #include "lsplit_kernels.cuh"
 #include "lsplit_pair.cuh"
 
@@ -227,7 +228,9 @@ __global__ void __launch_bounds__(256, 2) density_contract_tc_kernel(const float
 // psi_j = sum_n E2[j][n] T[j][n], one warp per point.  complex64: exact products
 // in pairs of floats, added up in pairs (2^-48 per addition) over 32 entries and
 // then in FP64; FP64 products of every entry were bound by the FP64 pipe (192 us
-// for 4096 x 2049, 45 us so).
+// for 4096 x 2049, 45 us so).  Entries of which the largest is not between 2^-90
+// and 2^100 take FP64 products: 64 of them could overflow a float, and below
+// 2^-102 a product loses its low part (E2 holds phases, at most 1).
 template <typename Real>
 __global__ void density_reduce_kernel(const typename CT<Real>::C* __restrict__ E2,
                                       const typename CT<Real>::C* __restrict__ T, int64_t nx, int64_t M2,
@@ -239,16 +242,27 @@ __global__ void density_reduce_kernel(const typename CT<Real>::C* __restrict__ E
   if constexpr (sizeof(Real) == 4) {
     for (int64_t n0 = lane; n0 < M2; n0 += 1024) {
       DF a{0.f, 0.f}, b{0.f, 0.f};
+      uint32_t mx = 0;
 #pragma unroll 4
       for (int64_t n = n0; n < M2 && n < n0 + 1024; n += 32) {
         const float2 e = E2[j * M2 + n], v = T[j * M2 + n];
+        mx = max(mx, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu));
         pair_mac(a, e.x, v.x);
         pair_mac(a, -e.y, v.y);
         pair_mac(b, e.x, v.y);
         pair_mac(b, e.y, v.x);
       }
-      re += (double)a.h + (double)a.l;
-      im += (double)b.h + (double)b.l;
+      constexpr uint32_t lo = (127u - 90u) << 23, hi = (127u + 100u) << 23;
+      if (mx == 0 || (mx >= lo && mx < hi)) {
+        re += (double)a.h + (double)a.l;
+        im += (double)b.h + (double)b.l;
+        continue;
+      }
+      for (int64_t n = n0; n < M2 && n < n0 + 1024; n += 32) {
+        const float2 e = E2[j * M2 + n], v = T[j * M2 + n];
+        re += (double)e.x * v.x - (double)e.y * v.y;
+        im += (double)e.x * v.y + (double)e.y * v.x;
+      }
     }
   } else {
     for (int64_t n = lane; n < M2; n += 32) {

@@ -58,3 +58,18 @@ def test_calls_of_several_threads(P, dtype):
     for t in threads:
         t.join()
     assert bad == []
+
+
+@pytest.mark.parametrize("exp", [-70, 90, 110, 121])
+def test_scaled_states(P, exp):
+    """The sum is linear: a state times a power of two gives the value times it,
+    up to the largest sums over m that complex64 holds (61 2^121; FP32 sums over
+    m, 1e-5 as in the parity tests).  All coefficients 1: near x = 0 the sum
+    over n adds up in one direction."""
+    p = W.bilayer_1d(30, 200, 1.0, 0.8, ecut=1e9)
+    ctx = P.Context(p, "c64")
+    phi = np.ones((p.M2, p.M1), dtype=np.complex128)
+    x = np.concatenate([[0.0], np.linspace(-1e-3, 1e-3, 70)])
+    want = ctx.density(ctx.from_dense(phi), x)
+    got = ctx.density(ctx.from_dense(phi * 2.0 ** exp), x) * 2.0 ** -exp
+    assert np.abs(got - want).max() < 1e-5 * np.abs(want).max()
