@@ -165,6 +165,7 @@ struct CachedTab {
   // (zero centre) and the logarithm of 1 + c'_0, the factor's scalar part
   std::shared_ptr<DevBuf> ipbuf;
   std::vector<cd> iptaps;
+  double l1 = 0;      // l1 norm of iptaps
   double tail = 0;    // l1 norm of the dropped taps
   std::complex<double> logdiag{0.0, 0.0};
 };
@@ -417,6 +418,7 @@ CachedTab stencil_table(ls_ctx* c, int layer, double s) {
         e.ipbuf = std::make_shared<DevBuf>();
         upload_c(c, *e.ipbuf, iptaps);
         e.iptaps = iptaps;
+        for (const cd& v : iptaps) e.l1 += std::abs(v);
         e.tail = tail;
         e.B = B;
         break;
@@ -932,6 +934,17 @@ double frame_decay(ls_ctx* c, int scheme, double tau) {
   return d >= std::log(0.0625) ? std::exp(d) : 0.0;
 }
 
+// The interaction frame of the stochastic complex64 calls evaluates the taps'
+// phases with the hardware sine and cosine (about 5e-7): below an FP32 rounding
+// of the result while the taps sum to no more than 0.15 (sampled factors last
+// frac_den times longer than deterministic ones).  Error of 20 Lie steps, lazy
+// phases and frame, by the sum: 0.12 9.9e-8 and 8.3e-8, 0.2 1.02e-7 and 1.09e-7,
+// 0.3 1.0e-7 and 1.5e-7, 0.5 1.1e-7 and 2.2e-7.
+bool sampled_frame(ls_ctx* c, int layer, double s) {
+  const CachedTab t = stencil_table(c, layer, s);
+  return t.B > 0 && t.l1 <= 0.15;
+}
+
 // Steps that one interaction-frame graph may hold.  The frame's state grows as
 // 1 / |Lambda| and Lambda is applied as 1 - (1 - |Lambda|): beyond |Lambda| =
 // 1/2 that cancels (and overflows in FP32 later), so a longer call runs as
@@ -1327,7 +1340,7 @@ void enqueue_step(ls_ctx* c, void* psi, int64_t n, double tau, int scheme, cudaS
   int npf = 0;
   lsk::SamplerArgs sa = sampler_args(c, scheme, npf);
   // Stochastic schemes in the interaction frame (complex64, every factor in the
-  // compact-kernel form): the kinetic factors act on every element, so the
+  // compact-kernel form with small taps): the kinetic factors act on every element, so the
   // frame is the same as the deterministic one; the sampled slices get their
   // factors, scalar parts included, and K(T) ends the call.  Otherwise the
   // pending phases are applied when a slice is sampled (touch times).
@@ -1335,7 +1348,7 @@ void enqueue_step(ls_ctx* c, void* psi, int64_t n, double tau, int scheme, cudaS
   for (size_t i = 0; i < ps.size() && sip; ++i) {
     const int64_t S = c->geom[ps[i].layer - 1].nslices;
     const int32_t p = std::max<int32_t>(1, (int32_t)(S / c->frac_den));
-    sip = stencil_table(c, ps[i].layer, ps[i].s * (double)S / (double)p).B > 0;
+    sip = sampled_frame(c, ps[i].layer, ps[i].s * (double)S / (double)p);
   }
   if (stoch) {
     if (!sip) {
@@ -2296,6 +2309,22 @@ void batch_units(int scheme, int32_t u[4][3][2], int& npass, double& unit, doubl
   }
 }
 
+// A stochastic complex64 call whose sampled factors all qualify for the frame
+// (the timeout test hook keeps the persistent kernel and its waits).
+bool batch_sampled_frame(ls_batch* b, double tau, int32_t scheme) {
+  if ((scheme != LS_LIE_STOCH && scheme != LS_STRANG_STOCH) || b->dtype != LS_C64 || b->unmet) return false;
+  std::vector<PassSpec> ps;
+  int32_t et = 0;
+  build_passes(scheme, tau, 1, ps, et);
+  for (ls_ctx* c : b->inst)
+    for (const PassSpec& q : ps) {
+      const int64_t S = c->geom[q.layer - 1].nslices;
+      const int32_t p = std::max<int32_t>(1, (int32_t)(S / c->frac_den));
+      if (!sampled_frame(c, q.layer, q.s * (double)S / (double)p)) return false;
+    }
+  return true;
+}
+
 // Capture the persistent launch of n steps on psi (tables uploaded first; the
 // graph keeps them alive).  The compact-only kernel (KIND 1) runs when every
 // factor of every instance takes the compact-kernel form.
@@ -2376,7 +2405,7 @@ std::unique_ptr<ls_batch::Cached> build_batch_graph(ls_batch* b, void* psi, int6
                     (scheme == LS_LIE || scheme == LS_STRANG || scheme == LS_STRANG_KP);
     // and so do the sampled slices of stochastic calls (launches per sub-step,
     // K(T) as their settle phase); the timeout test hook keeps the waits
-    const bool sip = kind == 1 && stoch && b->dtype == LS_C64 && !b->unmet;
+    const bool sip = kind == 1 && batch_sampled_frame(b, tau, scheme);
     size_t list_smem = 0;
     std::vector<cd> loglam(ninst, cd(0.0, 0.0));
     int32_t ip_step = 0;
@@ -2717,7 +2746,7 @@ std::string tune_key(const ls_batch* b, double tau, int32_t scheme) {
 // LSPLIT_STENCIL_CFG, or the timeout test hook armed.
 void maybe_tune(ls_batch* b, void* psi, int64_t n, double tau, int32_t scheme, cudaStream_t st) {
   if (!b->tune || b->unmet || b->dtype != LS_C64 || !batch_all_compact(b, tau, scheme)) return;
-  if (scheme == LS_LIE_STOCH || scheme == LS_STRANG_STOCH) return;   // launches per sub-step: nothing to choose
+  if (batch_sampled_frame(b, tau, scheme)) return;   // launches per sub-step: nothing to choose
   const std::string key = tune_key(b, tau, scheme);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
