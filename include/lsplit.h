@@ -285,7 +285,8 @@ int ls_batch_init_gaussian(ls_batch* batch, void* psi_dev, const double* x0_host
  * ls_step), the sampled-slice lists are drawn on the device in the same graph,
  * kinetic phases are applied lazily and a settle phase ends the call.
  * complex64 stochastic calls whose factors all take the compact-kernel form
- * with taps that sum to at most 0.15 run one launch per sub-step instead (in the same graph; no waits, so no
+ * with taps that sum to at most 0.15 run one launch per sub-step instead (in
+ * graphs of at most 3000 launches, replayed for longer calls; no waits, so no
  * LS_ERR_TIMEOUT, and nothing for the autotuner to choose).
  * Synchronises the stream to read the status: LS_ERR_TIMEOUT if a wait
  * expired (psi is then incomplete; the batch stays usable). */

@@ -80,3 +80,28 @@ def test_long_complex128_call_keeps_the_norm(P, monkeypatch, tiles, amp):
     ctx.step(psi, 20000, 1e-3, "strang")
     got, want = np.linalg.norm(ctx.to_dense(psi)), np.linalg.norm(x)
     assert abs(got / want - 1) < 4e-13
+
+
+@pytest.mark.parametrize("scheme", ["strang_stoch", "lie_stoch"])
+def test_long_stochastic_batch_in_pieces(P, scheme):
+    """Beyond one graph of launches a stochastic batched call is replayed in
+    pieces: same samples and states as the call cut anywhere, and device memory
+    that does not grow with the steps (64 MB: the graph of 60000 steps in one
+    piece holds 120000 or more launches)."""
+    import torch
+    probs = [W.bilayer_1d(9, 6, 2.0, 1.5, ecut=1e9), W.bilayer_1d(5, 12, 1.0, 0.7, ecut=1e9)]
+    b = P.Batch(probs, "c64")
+    xs = [W.random_state((p.M2, p.M1), 85 + i) for i, p in enumerate(probs)]
+    one, cut = b.empty(), b.empty()
+    for i, x in enumerate(xs):
+        b.set_dense(one, i, x)
+        b.set_dense(cut, i, x)
+    n = 3503
+    b.step(one, n, 1e-3, scheme, seed=4, step0=7)
+    b.step(cut, 1203, 1e-3, scheme, seed=4, step0=7)
+    b.step(cut, n - 1203, 1e-3, scheme, seed=4, step0=7 + 1203)
+    for i in range(2):
+        assert rel(b.get_dense(one, i), b.get_dense(cut, i)) < 2 * 3 * n * 2.0 ** -24
+    free = torch.cuda.mem_get_info()[0]
+    b.step(one, 60000, 1e-3, scheme, seed=4)
+    assert free - torch.cuda.mem_get_info()[0] < 64 << 20
