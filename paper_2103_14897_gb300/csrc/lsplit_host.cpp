@@ -211,6 +211,7 @@ struct ls_ctx {
   DevBuf tcplanes;                  // its split-BF16 DFT matrix planes
   DevBuf dir4, dir2;                // complex128 tile form: direction tables (built on first use)
   int sms = 0;
+  size_t block_max = 0;   // shared memory of a CTA (opt-in)
   int fast_variant = 0;   // shared-buffer / register-budget variant of the fast pass
   DevBuf tw[2], twb[2], bm[2], bp[2], chirp[2], vgrid[2];
   std::vector<double> vhost[2];
@@ -1150,6 +1151,8 @@ void enqueue_tiles(ls_ctx* c, void* psi, void* alt, int64_t n, double tau, int s
   in.psi = psi;
   in.alt = alt;
   const TilePlan x = tile_plan(c, scheme, tau, n, bv);
+  LS_CUDA(c->dtype == LS_C64 ? lsk::tile_prepare<float>(bv, x.e, c->block_max)
+                             : lsk::tile_prepare<double>(bv, x.e, c->block_max));
   for (lsk::TileArgs a : tile_passes(scheme, tau, n, bv, x.nf)) {
     a.tr = x.e - 2 * a.hr;
     a.tc = x.e - 2 * a.hc;
@@ -1765,6 +1768,7 @@ int ls_create(const ls_problem* prob, ls_ctx** out) {
       maxsm = (size_t)dev_max;
     }
     const size_t block_max = (size_t)dev_max + static_reserve;
+    c->block_max = block_max;
     if (c->dtype == LS_C64) LS_CUDA(lsk::pass_prepare<float>(block_max));
     else LS_CUDA(lsk::pass_prepare<double>(block_max));
     if (c->dtype == LS_C64) LS_CUDA(lsk::fast_prepare<float>(block_max));

@@ -210,6 +210,8 @@ struct TileArgs {
 // bv: 2 or 3 (complex64), 3, 4 or 5 (complex128); ext: rows and columns of a
 // tile with its halos, 32 (complex64), 16, 32 or 64 (complex128; not 16 with bv 5)
 template <typename Real> cudaError_t launch_tile(const TileArgs& a, int bv, int ext, int64_t ntiles, cudaStream_t st);
+// before an instance's first launch: its shared-memory limit (max_block per CTA)
+template <typename Real> cudaError_t tile_prepare(int bv, int ext, size_t max_block);
 // Tensor-core layer pass for contiguous 64 x 64 slices (complex64, MODE_STEP,
 // optionally the fused second factor in T2): the DFTs as split-BF16 matrix
 // products.  planes: 4 x 64 x 64 bf16 (row-major) with W[p][k] =

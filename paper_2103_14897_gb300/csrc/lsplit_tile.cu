@@ -821,36 +821,32 @@ __global__ void __launch_bounds__(RE * CE / (2 * SEG), MINB) tile_f32_kernel(con
   }
 }
 
-template <typename K> cudaError_t launch_k(K k, const TileArgs& a, int threads, size_t smem, int64_t ntiles,
-                                           cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(k, (unsigned)ntiles, threads, smem, st, a);
-}
+// Raise a kernel's shared-memory limit to the device's (the attribute belongs to
+// the process, so nothing may lower it again).
 template <int BV, int RE, int CE, int SEG, int MINB>
-cudaError_t launch_f32(const TileArgs& a, int64_t ntiles, cudaStream_t st) {
+cudaError_t launch_f32(const TileArgs* a, int64_t ntiles, size_t max_block, cudaStream_t st) {
   using Sh = TileShape<BV, RE, CE>;
+  const auto k = tile_f32_kernel<BV, RE, CE, SEG, MINB>;
+  if (!a) return allow_smem(k, max_block);
   const size_t smem = (size_t)2 * Sh::kElems * sizeof(float) +
-                      (size_t)a.nf * Sh::kAxis * (2 * BV * sizeof(float4) + sizeof(float2));
-  return launch_k(tile_f32_kernel<BV, RE, CE, SEG, MINB>, a, RE * CE / (2 * SEG), smem, ntiles, st);
+                      (size_t)a->nf * Sh::kAxis * (2 * BV * sizeof(float4) + sizeof(float2));
+  return launch_pdl(k, (unsigned)ntiles, RE * CE / (2 * SEG), smem, st, *a);
 }
 template <int BV, int RE, int CE, int SEG, int MINB>
-cudaError_t launch_f64(const TileArgs& a, int64_t ntiles, cudaStream_t st) {
+cudaError_t launch_f64(const TileArgs* a, int64_t ntiles, size_t max_block, cudaStream_t st) {
   using Sh = TileShape<BV, RE, CE>;
+  const auto k = tile_f64_kernel<BV, RE, CE, SEG, MINB>;
+  if (!a) return allow_smem(k, max_block);
   const size_t smem = (size_t)Sh::kElems * sizeof(double2) +
-                      (size_t)a.nf * Sh::kAxis * (Ar<double, BV>::kTabF4 + 1) * sizeof(float4);
-  return launch_k(tile_f64_kernel<BV, RE, CE, SEG, MINB>, a, RE * CE / SEG, smem, ntiles, st);
+                      (size_t)a->nf * Sh::kAxis * (Ar<double, BV>::kTabF4 + 1) * sizeof(float4);
+  return launch_pdl(k, (unsigned)ntiles, RE * CE / SEG, smem, st, *a);
 }
 
-}  // namespace
-
-template <typename Real> cudaError_t launch_tile(const TileArgs& a, int bv, int ext, int64_t ntiles, cudaStream_t st) {
-  if (ntiles <= 0) return cudaSuccess;
-  if (a.nf < 1 || a.nf > kTileMaxF || ntiles > 0x7fffffff || a.tr + 2 * a.hr > ext || a.tc + 2 * a.hc > ext ||
-      a.tr < 1 || a.tc < 1)
-    return cudaErrorInvalidValue;
+// The instance for bv and ext: launch it with *a, or (a NULL) prepare it.
+template <typename Real>
+cudaError_t tile_kernel(const TileArgs* a, int bv, int ext, int64_t ntiles, size_t max_block, cudaStream_t st) {
 #define LS_TILE(F, B, E, ...) \
-  if (bv == B && ext == E) return F<B, E, E, __VA_ARGS__>(a, ntiles, st);
+  if (bv == B && ext == E) return F<B, E, E, __VA_ARGS__>(a, ntiles, max_block, st);
   if constexpr (sizeof(Real) == 4) {
     LS_TILE(launch_f32, 2, 32, 2, 2)
     LS_TILE(launch_f32, 3, 32, 2, 2)
@@ -867,7 +863,22 @@ template <typename Real> cudaError_t launch_tile(const TileArgs& a, int bv, int 
 #undef LS_TILE
   return cudaErrorInvalidValue;
 }
+
+}  // namespace
+
+template <typename Real> cudaError_t launch_tile(const TileArgs& a, int bv, int ext, int64_t ntiles, cudaStream_t st) {
+  if (ntiles <= 0) return cudaSuccess;
+  if (a.nf < 1 || a.nf > kTileMaxF || ntiles > 0x7fffffff || a.tr + 2 * a.hr > ext || a.tc + 2 * a.hc > ext ||
+      a.tr < 1 || a.tc < 1)
+    return cudaErrorInvalidValue;
+  return tile_kernel<Real>(&a, bv, ext, ntiles, 0, st);
+}
+template <typename Real> cudaError_t tile_prepare(int bv, int ext, size_t max_block) {
+  return tile_kernel<Real>(nullptr, bv, ext, 0, max_block, nullptr);
+}
 template cudaError_t launch_tile<float>(const TileArgs&, int, int, int64_t, cudaStream_t);
 template cudaError_t launch_tile<double>(const TileArgs&, int, int, int64_t, cudaStream_t);
+template cudaError_t tile_prepare<float>(int, int, size_t);
+template cudaError_t tile_prepare<double>(int, int, size_t);
 
 }  // namespace lsk
