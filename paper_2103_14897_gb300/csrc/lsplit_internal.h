@@ -192,10 +192,7 @@ struct TileInst {
   float4 taps[2][2 * kTileMaxB + 1];  // per layer, tap d at kTileMaxB + d: (re hi, re lo, im hi, im lo)
 };
 struct TileArgs {
-  TileInst one;                       // a single instance (inst NULL), or
-  const TileInst* inst;               // ninst of them with cumulative tile counts
-  const int32_t* cum;
-  int32_t ninst;
+  TileInst one;
   int32_t nf;                         // factors of this pass
   int32_t layer[kTileMaxF];
   int64_t t[kTileMaxF];               // kinetic units before each factor, from the start of the call

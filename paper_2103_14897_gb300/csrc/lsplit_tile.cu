@@ -251,23 +251,14 @@ __device__ __forceinline__ int wraps(int a, int q) {
   return w;
 }
 
-// The tile of this CTA: instance, result rows [r0, r0 + vr) and columns
+// The tile of this CTA: result rows [r0, r0 + vr) and columns
 // [c0, c0 + vc), extents re x ce with the halos.
 struct TileGeo {
   const TileInst* in;
   int M1, M2, hr, hc, r0, c0, vr, vc, re, ce;
   __device__ __forceinline__ explicit TileGeo(const TileArgs& a) {
     in = &a.one;
-    int tile = blockIdx.x;
-    if (a.inst) {
-      int lo = 0, hi = a.ninst - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (a.cum[mid] <= tile) lo = mid; else hi = mid - 1;
-      }
-      in = a.inst + lo;
-      tile -= a.cum[lo];
-    }
+    const int tile = blockIdx.x;
     M1 = in->M1;
     M2 = in->M2;
     hr = a.hr;
