@@ -1097,7 +1097,18 @@ int64_t tile_count(const ls_ctx* c, const lsk::TileArgs& a) {
 struct TilePlan {
   int e = 0, nf = 0;
 };
+// (LSPLIT_TILE=extent,factors fixes both: with it every instance can be run on
+// any box; a pair that leaves a pass no result rows or columns is refused.)
 TilePlan tile_plan(const ls_ctx* c, int scheme, double tau, int64_t n, int bv) {
+  if (const char* ev = std::getenv("LSPLIT_TILE")) {
+    TilePlan x;
+    bool ok = std::sscanf(ev, "%d,%d", &x.e, &x.nf) == 2 && x.nf >= 1 && x.nf < lsk::kTileMaxF &&
+              (x.e == 32 || (c->dtype == LS_C128 && (x.e == 64 || (x.e == 16 && bv < 5))));
+    if (ok)
+      for (const lsk::TileArgs& a : tile_passes(scheme, tau, n, bv, x.nf)) ok = ok && x.e > 2 * a.hr && x.e > 2 * a.hc;
+    if (!ok) throw CudaError{cudaErrorInvalidValue, "LSPLIT_TILE"};
+    return x;
+  }
   if (c->dtype == LS_C64) return TilePlan{32, scheme == LS_STRANG ? 3 : 4};
   TilePlan best;
   double least = 0;
