@@ -746,6 +746,36 @@ int stencil_width(const lsk::LayerGeom& g, size_t esize, bool strided, size_t bu
   return (int)std::min<int64_t>(W, std::max<int64_t>(1, g.nslices));
 }
 
+// Rows per tile of the compact-kernel pass over all rows: the width with the
+// shortest time by a fit of measured times.  k tiles that share an SM take
+// t_k(w) = a_k w q / 1024 + b_k us; the busiest SM works off its tiles in
+// groups of as many as its registers hold (three, complex128 two).  Wider tiles
+// leave SMs idle on middle boxes and a nearly empty last group on large ones,
+// narrower ones pay b_k more often; within 1.5 %, the fit's own error, the
+// narrower (the groups do not end together, so more of them even out).  Strang,
+// 20 steps, us, widest and chosen: 401 x 401 334 (20 rows) and 205 (3), 641 x 641
+// 329 (13) and 234 (5), 1025 x 1025 355 (8) and 350 (4), 1401 x 1401 563 (6) and 524
+// (5), 1801 x 801 484 (4) and 426 (3), 2049 x 2049 956 (4) and 920 (2); over 39 boxes
+// the mean loss against the best width is 0.45 %.
+// Columns keep the widest (761 x 761: 338 with 8, 346 with 4).
+int stencil_rows(const ls_ctx* c) {
+  const bool f32 = c->dtype == LS_C64;
+  const int group = f32 ? 3 : 2, widest = c->stW[0];
+  const double a[3] = {f32 ? 0.50 : 0.55, f32 ? 0.89 : 1.0, 1.25}, b[3] = {f32 ? 0.70 : 0.10, f32 ? 0.87 : 0.15, 1.23};
+  const int64_t S = c->geom[0].nslices;
+  auto cost = [&](int w) {
+    const int64_t n = ((S + w - 1) / w + c->sms - 1) / c->sms;
+    const double e = (double)w * c->geom[0].qa / 1024.0;
+    auto t = [&](int k) { return a[k - 1] * e + b[k - 1]; };
+    return (double)(n / group) * t(group) + (n % group ? t((int)(n % group)) : 0.0);
+  };
+  double least = cost(1);
+  for (int w = 2; w <= widest; ++w) least = std::min(least, cost(w));
+  int w = 1;
+  while (cost(w) > 1.015 * least) ++w;
+  return w;
+}
+
 // Joint-cutoff predicate over the box (Sec. 3): fl(0.5 * fl(sum_i fl(u_i^2)))
 // <= Ec with u_i = sum_j fl(B1[i][j] m_j) + sum_j fl(B2[i][j] n_j) accumulated
 // left to right (this file is compiled without contraction).  mask may be
@@ -798,7 +828,10 @@ cudaError_t launch(ls_ctx* c, const lsk::PassArgs& a0, int L, int64_t nitems, cu
     return lsk::launch_tc2d(a0, c->tcplanes.p, (int)std::min<int64_t>(nitems, 2 * (int64_t)c->sms), st);
   if (a0.sB > 0 && (a0.mode == lsk::MODE_STEP || a0.mode == lsk::MODE_LAZY)) {
     lsk::PassArgs a = a0;
-    a.W = a.ip && a.list ? 1 : c->stW[L];   // sampled slices in the interaction frame: one per CTA
+    // sampled slices: in the interaction frame one per CTA; with lazy phases as
+    // many rows as still give every SM a CTA
+    a.W = a.ip && a.list ? 1 : c->stW[L];
+    if (a.list && !a.ip && L == 0) a.W = (int)std::max<int64_t>(1, std::min<int64_t>(a.W, nitems / c->sms));
     a.strided = (L == 1) ? 1 : 0;
     const int64_t ntiles = (nitems + a.W - 1) / a.W;
     if (c->dtype == LS_C64) return lsk::launch_stencil<float>(a, ntiles, st);
@@ -1791,25 +1824,7 @@ int ls_create(const ls_problem* prob, ls_ctx** out) {
     if (c->dtype == LS_C64) LS_CUDA(lsk::stencil_prepare<float>(block_max));
     else LS_CUDA(lsk::stencil_prepare<double>(block_max));
     for (int L = 0; L < 2; ++L) c->stW[L] = stencil_width(c->geom[L], c->esize, L == 1);
-    {
-      // rows: the width with the shortest time, waves of CTAs (three per SM) times
-      // the rows of a tile and about 1.5 rows' worth of tile overhead.  The widest
-      // tile leaves SMs idle on middle boxes and a nearly empty last wave on large
-      // ones: Strang, 20 steps, us, widest and chosen: 761 x 761 338 (10 rows) and
-      // 266 (3), 801 x 1801 542 (10) and 442 (4), 2049 x 2049 956 (4) and 945 (3).
-      // Columns keep the widest (761 x 761: 338 with 8, 346 with 4).
-      const int widest = c->stW[0];
-      const int64_t slots = 3 * (int64_t)c->sms, S = c->geom[0].nslices;
-      double least = 0;
-      for (int w = widest; w >= std::min(widest, 2); --w) {
-        const int64_t tiles = (S + w - 1) / w;
-        const double cost = (double)((tiles + slots - 1) / slots) * (w + 1.5);
-        if (w == widest || cost < least) {
-          least = cost;
-          c->stW[0] = w;
-        }
-      }
-    }
+    if (c->stW[0] > 0) c->stW[0] = stencil_rows(c.get());
     // tensor-core form of the contiguous 64 x 64 layer (complex64)
     if (c->dtype == LS_C64 && c->d == 2 && !c->p.shared && c->geom[0].qa == 64 && c->geom[0].qb == 64 &&
         lsk::tc2d_smem_bytes() + 8192 <= (size_t)dev_max + static_reserve && getenv_flag("LSPLIT_TC2D")) {
