@@ -1058,11 +1058,6 @@ int tile_instance(ls_ctx* c, int scheme, double tau, int64_t n, lsk::TileInst* i
   if (c->d != 1 || c->mask_mode != LS_MASK_INIT_ONLY || !tile_scheme(scheme, tau, ts) || getenv_flag("LSPLIT_NO_IP") ||
       getenv_flag("LSPLIT_NO_TILE"))
     return 0;
-  // complex64: where the in-place passes are bound by their launches.  Up to
-  // about four 32 x 32 tiles per SM the tile form is faster (Strang, 20 steps,
-  // us: 33 x 33 100 against 191, 257 x 257 121 / 328, 513 x 513 205 / 350),
-  // beyond the halos cost more than the launches (769 x 769 381 / 343).
-  if (c->dtype == LS_C64 && c->M1 * c->M2 > (int64_t)c->sms * 4 * 24 * 28) return 0;
   if (frame_decay(c, scheme, tau) == 0.0) return 0;
   lsk::TileInst in;
   std::memset(&in, 0, sizeof(in));
@@ -1074,6 +1069,20 @@ int tile_instance(ls_ctx* c, int scheme, double tau, int64_t n, lsk::TileInst* i
     if (b == 0) return 0;
     bv = std::max(bv, b);
     loglam += t.logdiag;
+  }
+  bv = std::max(bv, c->dtype == LS_C64 ? 2 : 3);
+  // complex64: where the in-place passes are bound by their launches, up to four
+  // tiles per SM (three for Strang with half-width 3); beyond, the halos cost more
+  // than the launches.  20 steps, us, tiles and in place; half-width 2, Strang:
+  // 401 x 401 120 / 204, 513 x 513 191 / 238, 609 x 609 222 / 227, 641 x 641 278 / 234; Lie:
+  // 401 x 401 78 / 150, 545 x 545 136 / 146, 577 x 577 166 / 151; half-width 3, Strang:
+  // 401 x 401 223 / 231, 545 x 545 275 / 240, 1025 x 257 268 / 227; Lie: 449 x 449
+  // 167 / 186, 545 x 545 232 / 168.  Long rows keep a few percent in place (2049 x
+  // 129: Strang 194 / 186, Lie 132 / 123).
+  if (c->dtype == LS_C64) {
+    const bool strang = scheme == LS_STRANG;
+    const int64_t tr = 32 - 2 * (strang ? bv : 2 * bv), tc = 32 - 4 * bv;
+    if (((c->M2 + tr - 1) / tr) * ((c->M1 + tc - 1) / tc) > (strang && bv == 3 ? 3 : 4) * (int64_t)c->sms) return 0;
   }
   if (inst) {
     lambda_parts((double)n * loglam, in.lam_turns, in.lam_def);
@@ -1087,7 +1096,7 @@ int tile_instance(ls_ctx* c, int scheme, double tau, int64_t n, lsk::TileInst* i
     in.X = c->geom[0].X_aa;
     *inst = in;
   }
-  return std::max(bv, c->dtype == LS_C64 ? 2 : 3);
+  return bv;
 }
 
 // The passes of n steps: an even number (the state ends in the caller's

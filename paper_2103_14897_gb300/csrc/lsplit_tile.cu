@@ -18,8 +18,8 @@
 //
 // What it is for.  complex64: boxes whose in-place passes are bound by their
 // launches; a pass of 3 or 4 factors on 32 x 32 tiles takes about 5 us, where
-// each factor's launch took 3 to 5 us (401 x 129, 50 Lie steps: 430 -> 170 us;
-// 513 x 513, 20 Strang steps: 350 -> 205 us).  complex128: every box (2049 x
+// each factor's launch takes 3 to 5 us (401 x 129, 50 Lie steps: 430 -> 170 us;
+// 20 Strang steps against in place: 257 x 257 113 / 172 us, 513 x 513 191 / 238 us).  complex128: every box (2049 x
 // 2049, 4 Strang steps: 6.56 -> 1.65 ms, at 65-70 % issue, about 570
 // instructions per element and factor; 65 x 65, 100 steps: 20.8 -> 1.47 ms, on
 // 16 x 16 tiles so that the box spreads over the SMs).
