@@ -197,10 +197,13 @@ int ls_init_gaussian(ls_ctx* ctx, void* psi_dev, const double* x0_host, double w
  * return.  With LS_MASK_PROJECT_EACH_STEP every step ends with the
  * projection onto the joint cutoff.  Deterministic 1D calls with short
  * potential kernels may alternate between psi_dev and a second array of the
- * same size that the library allocates (one per psi_dev with cached graphs,
- * freed with them; without memory for it the call runs in place).  Enqueued on stream (replays a cached CUDA
- * graph, one per (psi_dev, scheme, tau, nsteps); the graphs keep the tables
- * they use alive, and the table caches are bounded). */
+ * same size that the library allocates (one per psi_dev with cached graphs, at
+ * most eight per context, freed with them; without memory for it the call runs
+ * in place).  Enqueued on stream (replays a cached CUDA graph, one per (psi_dev,
+ * scheme, tau, nsteps); a deterministic call of so many steps that the factors'
+ * scalar parts would decay below 1/2 replays one of fewer steps and one of the
+ * rest; the graphs keep the tables they use alive, and the table caches are
+ * bounded). */
 int ls_step(ls_ctx* ctx, void* psi_dev, int64_t nsteps, double tau, int32_t scheme,
             uint64_t seed, uint64_t step0, void* stream);
 

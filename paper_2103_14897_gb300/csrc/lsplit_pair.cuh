@@ -1,7 +1,9 @@
 // Pairs of floats (an unevaluated sum of a high and a low part, about 2^-46
 // relative): the FP32 pipe of sm_103a runs at 64 times the FP64 rate, so a
 // pair operation of ten to twenty FP32 operations is the cheaper way to that
-// accuracy.  Explicit round-to-nearest intrinsics: nothing may be contracted.
+// accuracy.  Knuth's two-sum, Dekker's quick-two-sum, and products split by a
+// fused multiply-add.  Explicit round-to-nearest intrinsics: nothing may be
+// contracted.
 #pragma once
 namespace lsk {
 struct DF { float h, l; };

@@ -20,9 +20,9 @@
 // launches; a pass of 3 or 4 factors on 32 x 32 tiles takes about 5 us, where
 // each factor's launch takes 3 to 5 us (401 x 129, 50 Lie steps: 430 -> 170 us;
 // 20 Strang steps against in place: 257 x 257 113 / 172 us, 513 x 513 191 / 238 us).  complex128: every box (2049 x
-// 2049, 4 Strang steps: 6.56 -> 1.65 ms, at 65-70 % issue, about 570
-// instructions per element and factor; 65 x 65, 100 steps: 20.8 -> 1.47 ms, on
-// 16 x 16 tiles so that the box spreads over the SMs).
+// 2049, 4 Strang steps: 6.56 -> 1.62 ms, at 67 % issue, about 670 instructions
+// per element of a tile's extent and factor; 65 x 65, 100 steps: 20.8 -> 1.30 ms,
+// on 16 x 16 tiles so that the box spreads over the SMs).
 //
 // Sweep: a thread owns one line (row for layer 1, column for layer 2; lanes
 // take adjacent lines, the odd row pitch makes both free of bank conflicts)
@@ -33,13 +33,18 @@
 // complex64: 16 FMAs per tap pair and element, no phase evaluation in the
 // sweep; a thread takes two lines in the two lanes of paired FP32 operations
 // (real and imaginary parts in separate planes, the table entries doubled), so
-// that the FMA pipe and not the issue slots bounds it.  complex128: the FP64 pipe of sm_103a runs at 1/64 of the FP32 rate,
-// so only x + correction is formed in FP64 (two additions per component, the
-// rounding of the plain form); the correction, at most 2^-7 of its
-// neighbours, is formed in pairs of floats (about 2^-46 relative, 2^-53 and
-// less of the result) on the FP32 pipe, the taps |d| >= 3 (at most 2^-30) in
-// single floats.  The pairs are scaled by the tile's largest exponent, so the
-// whole FP64 range is taken.
+// that the FMA pipe and not the issue slots bounds it.  complex128: the FP64 pipe
+// of sm_103a runs at 1/64 of the FP32 rate, so only x + correction is formed in
+// FP64 (two additions per component, the rounding of the plain form); the
+// correction, at most 2^-7 of its neighbours, is formed in pairs of floats (about
+// 2^-46 relative, 2^-53 and less of the neighbours) on the FP32 pipe, the taps
+// |d| >= 3 (at most 2^-30) in single floats.  The pairs are scaled by the tile's
+// largest exponent, so the whole FP64 range is taken; neighbours below 2^-143 of
+// the largest count as zero.  The kinetic phases turn the taps from factor to
+// factor, so that their rounding does not add up: 33 x 25, Strang, error against
+// 80-bit arithmetic with the same kinetic phases, in place in FP64 and here: 100
+// steps 1.1e-14 and 1.3e-15, 1000 steps 1.1e-13 and 4.2e-15, 20000 steps 2.1e-12
+// and 3.7e-14 (tau max v = 3.4e-3; 2.5e-12 and 1.3e-12 at 1e-3).
 #include "lsplit_kernels.cuh"
 #include "lsplit_pair.cuh"
 
