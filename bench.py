@@ -570,7 +570,7 @@ def run_ours(args):
         bs.step(ps, NI, BATCH_TAU, "strang_stoch", seed=3)
         ts = _event_time_ms(lambda k: bs.step(ps, NI, BATCH_TAU, "strang_stoch", seed=3, step0=(k + 1) * NI), 5, st)
         subs["batch1d-256-strang_stoch"] = {"value": dof * NI * 5 / (ts / 1e3), "unit": "DOF-steps/s",
-                                            "note": "1/8 of the slices per sub-step (Algorithm 4), lazy kinetic phases"}
+                                            "note": "1/8 of the slices per sub-step (Algorithm 4), interaction frame"}
         del ps, bs
 
     if rank == 0:
