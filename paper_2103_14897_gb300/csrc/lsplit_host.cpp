@@ -3096,8 +3096,11 @@ int ls_batch_step(ls_batch* b, void* psi, int64_t n, double tau, int32_t scheme,
       LS_CUDA(cudaGraphLaunch(g->exec, st));
     };
     auto find = [&](int64_t m) -> ls_batch::Cached* {
-      for (auto& e : b->graphs)
-        if (e->psi == psi && e->scheme == scheme && e->tau == tau && e->n == m) return e.get();
+      for (auto it = b->graphs.begin(); it != b->graphs.end(); ++it)
+        if ((*it)->psi == psi && (*it)->scheme == scheme && (*it)->tau == tau && (*it)->n == m) {
+          b->graphs.splice(b->graphs.begin(), b->graphs, it);   // a later build evicts from the back
+          return b->graphs.front().get();
+        }
       return nullptr;
     };
     auto graph = [&](int64_t m) {

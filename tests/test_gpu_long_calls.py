@@ -105,3 +105,23 @@ def test_long_stochastic_batch_in_pieces(P, scheme):
     free = torch.cuda.mem_get_info()[0]
     b.step(one, 60000, 1e-3, scheme, seed=4)
     assert free - torch.cuda.mem_get_info()[0] < 64 << 20
+
+
+def test_pieces_with_a_full_list_of_graphs(P):
+    """The graph of a call's rest is the oldest of the batch's cached ones when
+    the graph of its pieces is built: it must not be the one that makes room."""
+    probs = [W.bilayer_1d(9, 6, 2.0, 1.5, ecut=1e9)]
+    b = P.Batch(probs, "c64")
+    x = W.random_state((probs[0].M2, probs[0].M1), 88)
+    psi, want = b.empty(), b.empty()
+    b.set_dense(psi, 0, x)
+    b.set_dense(want, 0, x)
+    steps = [11, 1, 2, 3, 1011]          # four cached graphs, the rest of 1011 = 1000 + 11 the oldest
+    step0 = 0
+    for n in steps:
+        b.step(psi, n, 1e-3, "strang_stoch", seed=5, step0=step0)
+        step0 += n
+    b2 = P.Batch(probs, "c64")
+    b2.step(want, 500, 1e-3, "strang_stoch", seed=5)
+    b2.step(want, step0 - 500, 1e-3, "strang_stoch", seed=5, step0=500)
+    assert rel(b.get_dense(psi, 0), b2.get_dense(want, 0)) < 2 * 3 * step0 * 2.0 ** -24
